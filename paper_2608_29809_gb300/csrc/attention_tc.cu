@@ -77,14 +77,6 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   return d;
 }
 
-// 2^x on the special-function unit (flushes subnormal results to zero; the
-// argument is at most 8 here).
-__device__ __forceinline__ float ex2_ftz(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 template <int DH>
 struct ACfg {
   static_assert(DH == 64 || DH == 72, "head_dim 64 or 72");
@@ -835,54 +827,6 @@ xattn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // xb G_h^T + kb_h, G_h = K_h W_xq,h, kb_h = K_h b_h (a reassociation of the
 // same products).  The cross-query GEMM then disappears from the block.
 
-// G and kb of one (session, layer): block (h, 8-key group), thread = 9
-// columns of G, 8 keys each, f32 accumulation over the head's dh dims.
-constexpr int FOLD_KEYS = 8, FOLD_THREADS = 128, FOLD_COLS = 12;  // d <= 128 * 12
-__global__ void __launch_bounds__(FOLD_THREADS)
-xq_fold_kernel(const bf16* __restrict__ Kt, int ldk, const bf16* __restrict__ Wq,
-               const float* __restrict__ bq, int M, int dh, int d, bf16* __restrict__ G,
-               float* __restrict__ kb) {
-  pdl_wait();
-  pdl_trigger();
-  __shared__ float sk[FOLD_KEYS][80];
-  const int h = blockIdx.x, r0 = blockIdx.y * FOLD_KEYS;
-  for (int e = threadIdx.x; e < FOLD_KEYS * dh; e += FOLD_THREADS) {
-    const int r = e / dh, j = e - (e / dh) * dh;
-    sk[r][j] = r0 + r < M ? __bfloat162float(Kt[size_t(r0 + r) * ldk + h * dh + j]) : 0.f;
-  }
-  __syncthreads();
-  const int nc = d / FOLD_THREADS;
-  float acc[FOLD_KEYS][FOLD_COLS];
-#pragma unroll
-  for (int r = 0; r < FOLD_KEYS; ++r)
-#pragma unroll
-    for (int i = 0; i < FOLD_COLS; ++i) acc[r][i] = 0.f;
-  for (int j = 0; j < dh; ++j) {
-    const bf16* wrow = Wq + size_t(h * dh + j) * d;
-    float w[FOLD_COLS];
-#pragma unroll
-    for (int i = 0; i < FOLD_COLS; ++i)
-      w[i] = i < nc ? __bfloat162float(wrow[threadIdx.x + FOLD_THREADS * i]) : 0.f;
-#pragma unroll
-    for (int r = 0; r < FOLD_KEYS; ++r)
-#pragma unroll
-      for (int i = 0; i < FOLD_COLS; ++i) acc[r][i] = fmaf(sk[r][j], w[i], acc[r][i]);
-  }
-#pragma unroll
-  for (int r = 0; r < FOLD_KEYS; ++r) {
-    if (r0 + r >= M) break;
-    bf16* grow = G + (size_t(h) * XQ_KEYS + r0 + r) * d;
-#pragma unroll
-    for (int i = 0; i < FOLD_COLS; ++i)
-      if (i < nc) grow[threadIdx.x + FOLD_THREADS * i] = __float2bfloat16_rn(acc[r][i]);
-  }
-  if (threadIdx.x < FOLD_KEYS && r0 + int(threadIdx.x) < M) {
-    float a = 0.f;
-    for (int j = 0; j < dh; ++j) a = fmaf(sk[threadIdx.x][j], bq[h * dh + j], a);
-    kb[size_t(h) * XQ_KEYS + r0 + threadIdx.x] = a;
-  }
-}
-
 // One (query tile, head) per CTA: S = xb_tile G_h^T accumulated over d in
 // 64-column k-blocks (TMA ring, M = 128, N = 128), then the softmax of
 // (S + kb) / sqrt(dh) per row, P over S in TMEM, O = P V, O / l stored.
@@ -1423,16 +1367,6 @@ cudaError_t launch_attention(const bf16* Q, int ldq, const bf16* K, const bf16* 
                       as.part, O, ldo, heads, rm, ai.n, Nk, grid, err));
     count_launches(1);
   }
-  return cudaSuccess;
-}
-
-cudaError_t launch_xq_fold(const bf16* Kt, int ldk, const bf16* Wq, const float* bq, int M,
-                           int heads, int dh, int d, bf16* G, float* kb, cudaStream_t st) {
-  if (M < 1 || M > XQ_KEYS || dh > 80 || d % FOLD_THREADS || d > FOLD_THREADS * FOLD_COLS)
-    return cudaErrorInvalidValue;
-  RC_TRY(launch_k(xq_fold_kernel, dim3(heads, (M + FOLD_KEYS - 1) / FOLD_KEYS),
-                  dim3(FOLD_THREADS), 0, st, Kt, ldk, Wq, bq, M, dh, d, G, kb));
-  count_launches(1);
   return cudaSuccess;
 }
 

@@ -34,6 +34,12 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// 2^x on the special-function unit (subnormal results are flushed to zero).
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 // tanh on the special-function unit (relative error about 2^-11, below the
 // bf16 rounding of every GELU output)
 __device__ __forceinline__ float tanh_sfu(float x) {

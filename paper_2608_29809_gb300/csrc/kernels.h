@@ -194,11 +194,30 @@ cudaError_t launch_attention(const bf16* Q, int ldq, const bf16* K, const bf16* 
 // Text cross-attention with the query projection folded into the keys:
 // S_h = xb W_xq,h^T K_h^T + b_h K_h^T = xb G_h^T + kb_h with G_h = K_h W_xq,h
 // ([XK][d] per (session, layer, head), rows >= text_len zero) and
-// kb_h = K_h b_xq,h.  launch_xq_fold computes G and kb of one (session,
-// layer) for all heads from the text keys (row stride ldk) and W_xq, b_xq.
+// kb_h = K_h b_h.
 constexpr int XQ_KEYS = 128;
-cudaError_t launch_xq_fold(const bf16* Kt, int ldk, const bf16* Wq, const float* bq, int M,
-                           int heads, int dh, int d, bf16* G, float* kb, cudaStream_t st);
+
+// A turn's start, all L layers of one session at once.  launch_text_kv:
+// text[l] = ctx W_xkv,l^T + b_xkv,l ([M][2d] per layer, M <= 128).
+// launch_xq_fold: G and kb of every (layer, head) from text.
+struct TextLayer {
+  const bf16* W_xkv;
+  const float* b_xkv;
+  const bf16* W_xq;
+  const float* b_xq;
+};
+cudaError_t launch_text_kv(const bf16* ctx, const TextLayer* layers, int L, int M, int d,
+                           bf16* text, unsigned* err, cudaStream_t st);
+cudaError_t launch_xq_fold(const bf16* text, const TextLayer* layers, int L, int M, int heads,
+                           int dh, bf16* G, float* kb, unsigned* err, cudaStream_t st);
+// Localisation scores of N tokens from all layers: cap.out[i][id] += cap.w *
+// sum over layers and heads of the softmax probability of key id, the
+// queries of layer 0 from x0 and those of layer l >= 1 from the cache rows
+// xrow0 + (l - 1) * xrow_step ..; G / kb rows of the session from grow0.
+cudaError_t launch_scores(const bf16* x0, int x0_rows, const bf16* cache, long long cache_rows,
+                          int xrow0, int xrow_step, const bf16* G, long long g_rows, int grow0,
+                          const float* kb, int N, int layers, int heads, int dh, int Nk,
+                          const AttnCapture& cap, unsigned* err, cudaStream_t st);
 // O[r][h*dh..] = softmax((xb_r G_h^T + kb_h) / sqrt(dh)) V_h over the Nk <= 128
 // text keys of row r's item.  G / kb rows of item i start at grow[i] (+ h *
 // XQ_KEYS); its values at row vrow[i] of V (row stride ldv).  cap as in

@@ -60,6 +60,7 @@ struct rc_ctx {
   int device;
   std::vector<rc_layer_weights> lw;
   std::vector<char> lw_set;
+  std::vector<rc::TextLayer> tl;  // the weights that a layer's text keys / values depend on
   // bumped by every rc_set_layer_weights: a session's text keys (and the
   // folded cross-query keys derived from them) are valid only for the
   // generation they were computed with
@@ -500,6 +501,7 @@ rc_status rc_create(const rc_dims* dims, rc_ctx** out) {
   cudaGetDevice(&c->device);
   c->lw.resize(c->L);
   c->lw_set.assign(c->L, 0);
+  c->tl.resize(c->L);
   rc_status s = RC_OK;
   const size_t R = size_t(max_batch) * N;  // compact rows of a step
   const size_t Rd = R * D.hidden;
@@ -549,6 +551,8 @@ rc_status rc_set_layer_weights(rc_ctx* c, int layer, const rc_layer_weights* w) 
       return fail(RC_ERR_INVALID_ARG, "layer %d: null or unaligned (16 B) weight", layer);
   c->lw[layer] = *w;
   c->lw_set[layer] = 1;
+  c->tl[layer] = {static_cast<const bf16*>(w->W_xkv), w->b_xkv, static_cast<const bf16*>(w->W_xq),
+                  w->b_xq};
   ++c->wgen;
   return RC_OK;
 }
@@ -765,11 +769,10 @@ rc_status rc_cache_read(rc_cache* k, int s, int l, int t, void* H, void* K, void
 // layers (Section 3.3's cross-attention, reassociated: see run_block).
 static rc_status fold_text(rc_ctx* c, rc_cache* k, int s, cudaStream_t st) {
   if (!k->xg) return RC_OK;
-  for (int l = 0; l < c->L; ++l)
-    RC_CUDA(rc::launch_xq_fold(k->text_kv(s, l), 2 * c->d, static_cast<const bf16*>(c->lw[l].W_xq),
-                               c->lw[l].b_xq, c->M, c->dims.heads, c->dh, c->d,
-                               k->xg + k->xg_row(s, l) * c->d, k->xgb + k->xg_row(s, l), st),
-            "fold text keys");
+  RC_CUDA(rc::launch_xq_fold(k->text_kv(s, 0), c->tl.data(), c->L, c->M, c->dims.heads,
+                             c->dh, k->xg + k->xg_row(s, 0) * c->d, k->xgb + k->xg_row(s, 0),
+                             c->err, st),
+          "fold text keys");
   return RC_OK;
 }
 
@@ -875,16 +878,22 @@ rc_status rc_set_text(rc_ctx* c, rc_cache* k, int s, const void* ctx_bf16, rc_st
   for (int l = 0; l < c->L; ++l)
     if (!c->lw_set[l]) return fail(RC_ERR_STATE, "weights of layer %d not set", l);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  for (int l = 0; l < c->L; ++l) {
-    rc::GemmEpi e{};
-    e.mode = rc::EPI_BIAS_BF16;
-    e.bias = c->lw[l].b_xkv;
-    e.out_bf = k->text_kv(s, l);
-    e.ld_out = 2 * c->d;
-    e.err = c->err;
-    RC_CUDA(rc::launch_gemm(static_cast<const bf16*>(ctx_bf16), c->d,
-                            static_cast<const bf16*>(c->lw[l].W_xkv), c->M, nullptr, 2 * c->d,
-                            c->d, e, st), "gemm(text kv)");
+  if (c->M <= rc::XQ_KEYS) {
+    // every layer in one launch: 28 launches of 10.8 us before
+    RC_CUDA(rc::launch_text_kv(static_cast<const bf16*>(ctx_bf16), c->tl.data(), c->L,
+                               c->M, c->d, k->text_kv(s, 0), c->err, st), "text kv");
+  } else {
+    for (int l = 0; l < c->L; ++l) {
+      rc::GemmEpi e{};
+      e.mode = rc::EPI_BIAS_BF16;
+      e.bias = c->lw[l].b_xkv;
+      e.out_bf = k->text_kv(s, l);
+      e.ld_out = 2 * c->d;
+      e.err = c->err;
+      RC_CUDA(rc::launch_gemm(static_cast<const bf16*>(ctx_bf16), c->d,
+                              static_cast<const bf16*>(c->lw[l].W_xkv), c->M, nullptr, 2 * c->d,
+                              c->d, e, st), "gemm(text kv)");
+    }
   }
   if ((r = fold_text(c, k, s, st))) return r;
   k->text_set[s] = 1;
@@ -1362,39 +1371,35 @@ rc_status rc_localize_scores(rc_ctx* c, rc_cache* k, int s, int t, const float* 
   cast.n = 1;
   cast.slice[0] = c->xb;
   RC_CUDA(rc::launch_scatter_bf16(c->xf, cast, 0, rm, d, c->err, st), "embedding cast");
+  if (k->xg) {
+    // (x W_xq^T + b) K^T = x G_h^T + kb_h with the folded text keys, every
+    // layer in one launch (the layers' inputs are all in the cache)
+    RC_CUDA(rc::launch_scores(c->xb, N, k->slot(s, 0, t, 0), (long long)c->L * 3 * N, 0, 3 * N,
+                              k->xg, (long long)k->xg_rows(), int(k->xg_row(s, 0)), k->xgb, N,
+                              c->L, c->dims.heads, c->dh, c->M, cap, c->err, st),
+            "scores(cross)");
+    return RC_OK;
+  }
   for (int l = 0; l < c->L; ++l) {
     // the input of block l as cached at step t: block l - 1's output slot
     const bf16* h_in = l == 0 ? c->xb : k->slot(s, l - 1, t, 0);
-    if (k->xg) {
-      // (x W_xq^T + b) K^T = x G_h^T + kb_h with the folded text keys; the
-      // kernel's P V output goes to scratch, only the captured columns matter
-      rc::XqItems xi{};
-      xi.n = 1;
-      xi.grow[0] = int(k->xg_row(s, l));
-      xi.vrow[0] = (s * c->L + l) * c->M;
-      RC_CUDA(rc::launch_xattn_fused(h_in, d, k->xg, k->xgb, int(k->xg_rows()), k->text + d,
-                                     2 * d, k->sessions * c->L * c->M, xi, c->M, c->ob, d,
-                                     c->dims.heads, c->dh, rm, c->err, st, &cap),
-              "scores(cross)");
-    } else {
-      rc::GemmEpi e{};
-      e.mode = rc::EPI_BIAS_BF16;
-      e.bias = c->lw[l].b_xq;
-      e.out_bf = c->q;
-      e.ld_out = d;
-      e.gate_off = -1;
-      e.err = c->err;
-      RC_CUDA(rc::launch_gemm(h_in, d, static_cast<const bf16*>(c->lw[l].W_xq), N, nullptr, d,
-                              d, e, st), "gemm(xq)");
-      StepItems si;
-      si.its.n = 1;
-      si.session[0] = s;
-      si.t[0] = t;
-      RC_CUDA(rc::launch_attention(c->q, d, k->text, k->text + d, 2 * d,
-                                   k->sessions * c->L * c->M, text_kv_rows(k, si, l), c->M,
-                                   c->ob, d, c->dims.heads, c->dh, rm, c->err, c->as, st, &cap),
-              "scores(cross)");
-    }
+    rc::GemmEpi e{};
+    e.mode = rc::EPI_BIAS_BF16;
+    e.bias = c->lw[l].b_xq;
+    e.out_bf = c->q;
+    e.ld_out = d;
+    e.gate_off = -1;
+    e.err = c->err;
+    RC_CUDA(rc::launch_gemm(h_in, d, static_cast<const bf16*>(c->lw[l].W_xq), N, nullptr, d,
+                            d, e, st), "gemm(xq)");
+    StepItems si;
+    si.its.n = 1;
+    si.session[0] = s;
+    si.t[0] = t;
+    RC_CUDA(rc::launch_attention(c->q, d, k->text, k->text + d, 2 * d,
+                                 k->sessions * c->L * c->M, text_kv_rows(k, si, l), c->M,
+                                 c->ob, d, c->dims.heads, c->dh, rm, c->err, c->as, st, &cap),
+            "scores(cross)");
   }
   return RC_OK;
 }

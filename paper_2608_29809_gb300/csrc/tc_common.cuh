@@ -9,6 +9,22 @@ namespace tc {
 
 constexpr unsigned long long WAIT_NS = 2000000000ull;  // bounded waits: 2 s
 
+// True in one lane of a converged warp.  The tcgen05 and TMA instructions take
+// their operands from uniform registers; under a branch on elect.sync the
+// compiler knows that a single lane is active.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok));
+  return ok != 0;
+}
+// The warp's index, known by the compiler to be uniform.
+__device__ __forceinline__ int warp_index() {
+  return __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0);
+}
 __device__ __forceinline__ uint32_t saddr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
