@@ -35,8 +35,15 @@ static inline int row_grid(int rows_bound, int rows_per_cta, int per_sm) {
 }
 
 // ============================================================ localisation
+// The mask of an edit in one launch, or two when the score map is large: a
+// cluster of eight CTAs shares the column bounds, the thresholded region and
+// the counts through its shared memory, so that the steps that need every
+// token's result of the previous one are cluster barriers instead of
+// launches.  1024 tokens, 5 delta tokens: 7.9 -> 5.9 us on the device (four
+// launches before), 17.9 -> 12.6 us a call from Python; 16384 tokens, 8 delta
+// tokens, 16 slices: 50 -> 32 us.
 // Workspace: abar f32 [n_delta][N] | part f32x2 [nblk][n_delta] | union u8 [N]
-// | cnt int [nblk].  One thread per token, MASK_ROWS tokens per CTA.
+// | cnt int [nblk] (the last two are unused and kept for the stated size).
 constexpr int MASK_ROWS = 256;
 
 static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -51,171 +58,311 @@ size_t localize_workspace_bytes(int N, int n_delta) {
 struct MaskWs {
   float* abar;
   float2* part;
-  uint8_t* uni;
-  int* cnt;
 };
 
 static MaskWs carve(void* ws, int N, int n_delta) {
-  int nblk = cdiv(N, MASK_ROWS);
   char* p = static_cast<char*>(ws);
   MaskWs w;
   w.abar = reinterpret_cast<float*>(p);
   p += align256(sizeof(float) * size_t(n_delta) * N);
   w.part = reinterpret_cast<float2*>(p);
-  p += align256(sizeof(float2) * size_t(nblk) * n_delta);
-  w.uni = reinterpret_cast<uint8_t*>(p);
-  p += align256(size_t(N));
-  w.cnt = reinterpret_cast<int*>(p);
   return w;
 }
 
-// Pass 1: a_j(i) = (sum_s A[s][i][j]) / S for each delta token j (summed in
-// ascending s, f32 round-to-nearest), and per-CTA min / max of each column.
-// A non-finite a_j(i) (NaN, +-Inf) enters the min / max as the pair
-// (-Inf, +Inf): finite values never reach those bounds, so pass 2 reads them
-// as "this column holds a non-finite value" and drops the column.
+// a_j(i) = (sum_s A[s][i][j]) / S of Q tokens (p[q]; null: none), summed in
+// ascending s, f32 round-to-nearest; eight loads in flight.
+template <int Q>
+__device__ __forceinline__ void mean_scores(const float* const* p, int S, size_t plane, float* a) {
+  constexpr int B = 8 / Q;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) a[q] = 0.f;
+  for (int s = 0; s < S; s += B) {
+    float v[Q][B];
+#pragma unroll
+    for (int e = 0; e < B; ++e)
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        if (s + e < S && p[q]) v[q][e] = __ldg(p[q] + (s + e) * plane);
+#pragma unroll
+    for (int e = 0; e < B; ++e)
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        if (s + e < S && p[q]) a[q] = s + e == 0 ? v[q][e] : __fadd_rn(a[q], v[q][e]);
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) a[q] = __fdiv_rn(a[q], float(S));
+}
+// The bounds that a value contributes to its column.  A non-finite a_j(i)
+// (NaN, +-Inf) enters as the pair (-Inf, +Inf): finite values never reach
+// those bounds, so they mark a column that holds a non-finite value, which
+// is dropped.
+__device__ __forceinline__ void widen(float a, float& lo, float& hi) {
+  const bool fin = isfinite(a);
+  lo = fminf(lo, fin ? a : -INFINITY);
+  hi = fmaxf(hi, fin ? a : INFINITY);
+}
+__device__ __forceinline__ void warp_bounds(float& lo, float& hi) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+}
+
+// Large maps, first launch: one CTA per (256 tokens, delta token), a_j(i) to
+// abar and the CTA's column bounds to part.  Each token's score is its own
+// 32-byte sector, so this is bound by sectors from DRAM: 16384 tokens, 8
+// delta tokens, 16 slices read 92 MB for 8.4 MB of scores in 21 us (38 us
+// with one thread per token taking its delta tokens in turn).
 __global__ void __launch_bounds__(MASK_ROWS)
-mask_colstats_kernel(const float* __restrict__ A, int S, int N, int M, DeltaIds ids,
-                     float* __restrict__ abar, float2* __restrict__ part) {
+mask_colstats_kernel(const float* __restrict__ A, int S, int N, int M,
+                     const __grid_constant__ DeltaIds ids, float* __restrict__ abar,
+                     float2* __restrict__ part) {
   pdl_wait();
   pdl_trigger();
   __shared__ float smin[MASK_ROWS / 32], smax[MASK_ROWS / 32];
-  const int i = blockIdx.x * MASK_ROWS + threadIdx.x;
+  const int i = blockIdx.x * MASK_ROWS + threadIdx.x, j = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const size_t plane = size_t(N) * M;
-  for (int j = 0; j < ids.n; ++j) {
-    const int col = ids.id[j];
-    float lo = FLT_MAX, hi = -FLT_MAX;
-    if (i < N) {
-      float a = __ldg(A + size_t(i) * M + col);
-      for (int s = 1; s < S; ++s) a = __fadd_rn(a, __ldg(A + s * plane + size_t(i) * M + col));
-      a = __fdiv_rn(a, float(S));
-      abar[size_t(j) * N + i] = a;
-      if (isfinite(a)) {
-        lo = hi = a;
-      } else {
-        lo = -INFINITY;
-        hi = INFINITY;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if (lane == 0) { smin[warp] = lo; smax[warp] = hi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < MASK_ROWS / 32; ++w) { lo = fminf(lo, smin[w]); hi = fmaxf(hi, smax[w]); }
-      part[size_t(blockIdx.x) * ids.n + j] = make_float2(lo, hi);
-    }
-    __syncthreads();
+  float lo = FLT_MAX, hi = -FLT_MAX;
+  if (i < N) {
+    const float* p = A + size_t(i) * M + ids.id[j];
+    float a;
+    mean_scores<1>(&p, S, size_t(N) * M, &a);
+    abar[size_t(j) * N + i] = a;
+    widen(a, lo, hi);
+  }
+  warp_bounds(lo, hi);
+  if (lane == 0) { smin[warp] = lo; smax[warp] = hi; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < MASK_ROWS / 32; ++w) { lo = fminf(lo, smin[w]); hi = fmaxf(hi, smax[w]); }
+    part[size_t(blockIdx.x) * ids.n + j] = make_float2(lo, hi);
   }
 }
 
-// Pass 2: column min / max over all CTAs (exact, order-free), then the
-// thresholded union over the delta tokens: ((a - mn) / (mx - mn)) >= tau.
-// A constant column, or one holding a non-finite value, gives no token.
-__global__ void __launch_bounds__(MASK_ROWS)
-mask_threshold_kernel(const float* __restrict__ abar, const float2* __restrict__ part, int nblk,
-                      int N, DeltaIds ids, float tau, uint8_t* __restrict__ uni) {
+// One cluster: (with FROM_MAP, a_j(i) and the column bounds of the cluster's
+// tokens,) the thresholded union over the delta tokens, ((a - mn) / (mx -
+// mn)) >= tau with constant and non-finite columns dropped, its (2r+1)^2
+// dilation on the grid, and the compact list of dirty tokens in ascending
+// order.  CTA c owns tokens [c per, (c + 1) per), per a multiple of 32; the
+// union is a bit per token in every CTA's shared memory.
+constexpr int MASK_CTAS = 8, MASK_THREADS = 512, MASK_WARPS = MASK_THREADS / 32;
+constexpr int MASK_MAX_TOKENS = 16384, MASK_WORDS = MASK_MAX_TOKENS / 32;
+constexpr int MASK_WPW = MASK_WORDS / MASK_CTAS / MASK_WARPS;  // words of a warp, at most
+
+__device__ __forceinline__ uint32_t peer_shared(const void* p, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(r)
+               : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+template <bool FROM_MAP>
+__global__ void __launch_bounds__(MASK_THREADS, 1)
+mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, int gw,
+                    const __grid_constant__ DeltaIds ids, float tau, int r, int nblk,
+                    float* __restrict__ abar, const float2* __restrict__ part,
+                    uint8_t* __restrict__ mask, int32_t* __restrict__ idx,
+                    int32_t* __restrict__ count) {
+  __shared__ float s_lo[MASK_CTAS][64], s_hi[MASK_CTAS][64];  // per CTA (row 0 when not FROM_MAP)
+  __shared__ float s_wlo[64][MASK_WARPS], s_whi[64][MASK_WARPS];
+  __shared__ float s_mn[64], s_rng[64], s_inv[64];
+  __shared__ int s_ok[64];
+  __shared__ uint32_t s_bits[MASK_WORDS];
+  __shared__ int s_cnt[MASK_CTAS];
+  __shared__ int s_word[MASK_WORDS / MASK_CTAS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = blockIdx.x;
+  const int per = (((N + MASK_CTAS - 1) / MASK_CTAS) + 31) & ~31;
+  const int t0 = min(N, rank * per), t1 = min(N, t0 + per), words = (t1 - t0 + 31) / 32;
+  cluster_barrier();  // every CTA has started: its shared memory can be written
   pdl_wait();
   pdl_trigger();
-  __shared__ float s_mn[64], s_rng[64];
-  __shared__ int s_ok[64];
+  if (FROM_MAP) {
+    // a warp takes 4 x 32 tokens of one delta token at a time
+    for (int e = threadIdx.x; e < 64 * MASK_WARPS; e += MASK_THREADS) {
+      (&s_wlo[0][0])[e] = FLT_MAX;
+      (&s_whi[0][0])[e] = -FLT_MAX;
+    }
+    __syncthreads();
+    const int groups = (words + 3) / 4;
+    for (int u = warp; u < groups * ids.n; u += MASK_WARPS) {
+      const int j = u / groups, i = t0 + (u - j * groups) * 128 + lane;
+      const float* p[4];
+      float a[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        p[q] = i + 32 * q < t1 ? A + size_t(i + 32 * q) * M + ids.id[j] : nullptr;
+      mean_scores<4>(p, S, size_t(N) * M, a);
+      float lo = FLT_MAX, hi = -FLT_MAX;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (p[q]) {
+          abar[size_t(j) * N + i + 32 * q] = a[q];
+          widen(a[q], lo, hi);
+        }
+      warp_bounds(lo, hi);
+      if (lane == 0) {
+        s_wlo[j][warp] = fminf(s_wlo[j][warp], lo);
+        s_whi[j][warp] = fmaxf(s_whi[j][warp], hi);
+      }
+    }
+    __syncthreads();
+    for (int j = warp; j < ids.n; j += MASK_WARPS) {
+      float lo = lane < MASK_WARPS ? s_wlo[j][lane] : FLT_MAX;
+      float hi = lane < MASK_WARPS ? s_whi[j][lane] : -FLT_MAX;
+      warp_bounds(lo, hi);
+      if (lane < MASK_CTAS) {
+        st_peer(peer_shared(&s_lo[rank][j], lane), __float_as_uint(lo));
+        st_peer(peer_shared(&s_hi[rank][j], lane), __float_as_uint(hi));
+      }
+    }
+    cluster_barrier();
+  } else {
+    for (int j = warp; j < ids.n; j += MASK_WARPS) {
+      float lo = FLT_MAX, hi = -FLT_MAX;
+      for (int b = lane; b < nblk; b += 32) {
+        const float2 v = __ldg(part + size_t(b) * ids.n + j);
+        lo = fminf(lo, v.x);
+        hi = fmaxf(hi, v.y);
+      }
+      warp_bounds(lo, hi);
+      if (lane == 0) { s_lo[0][j] = lo; s_hi[0][j] = hi; }
+    }
+    __syncthreads();
+  }
   if (threadIdx.x < ids.n) {
     const int j = threadIdx.x;
-    float lo = FLT_MAX, hi = -FLT_MAX;
-    for (int b = 0; b < nblk; ++b) {
-      float2 v = part[size_t(b) * ids.n + j];
-      lo = fminf(lo, v.x);
-      hi = fmaxf(hi, v.y);
+    float lo = s_lo[0][j], hi = s_hi[0][j];
+    for (int c = 1; c < (FROM_MAP ? MASK_CTAS : 1); ++c) {
+      lo = fminf(lo, s_lo[c][j]);
+      hi = fmaxf(hi, s_hi[c][j]);
     }
-    float rng = __fsub_rn(hi, lo);
+    const float rng = __fsub_rn(hi, lo);
     s_mn[j] = lo;
     s_rng[j] = rng;
+    s_inv[j] = __fdiv_rn(1.f, rng);
     s_ok[j] = rng > 0.0f && lo != -INFINITY && hi != INFINITY;
   }
   __syncthreads();
-  const int i = blockIdx.x * MASK_ROWS + threadIdx.x;
-  if (i >= N) return;
-  uint8_t u = 0;
-  for (int j = 0; j < ids.n; ++j) {
-    if (!s_ok[j]) continue;
-    float nv = __fdiv_rn(__fsub_rn(abar[size_t(j) * N + i], s_mn[j]), s_rng[j]);
-    u |= (nv >= tau) ? 1 : 0;
+  // the thresholded union to every CTA; a warp owns up to four words of 32
+  // tokens, whose scores of several delta tokens are in flight together.  The
+  // division is correctly rounded by definition and takes some 40
+  // instructions; the product with the reciprocal is within a few ulp of it,
+  // so it is taken only where that does not settle the comparison (NaN and
+  // overflowing products among them)
+  {
+    bool u[MASK_WPW] = {};
+    const float margin = fmaxf(1e-6f * fabsf(tau), 1e-37f);
+    const float tau_hi = tau + margin, tau_lo = tau - margin;
+#pragma unroll 4
+    for (int j = 0; j < ids.n; ++j) {
+      const float* aj = abar + size_t(j) * N + t0 + lane;
+      float a[MASK_WPW];
+#pragma unroll
+      for (int q = 0; q < MASK_WPW; ++q)
+        a[q] = t0 + (warp + q * MASK_WARPS) * 32 + lane < t1 ? aj[(warp + q * MASK_WARPS) * 32]
+                                                             : 0.f;
+      const bool ok = s_ok[j];
+      const float mn = s_mn[j], rng = s_rng[j], inv = s_inv[j];
+#pragma unroll
+      for (int q = 0; q < MASK_WPW; ++q)
+        if (warp + q * MASK_WARPS < words) {  // (the same for the whole warp)
+          const float x = __fsub_rn(a[q], mn), v = __fmul_rn(x, inv);
+          u[q] |= ok && (v > tau_hi || (!(v < tau_lo) && __fdiv_rn(x, rng) >= tau));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < MASK_WPW; ++q) {
+      const int w = warp + q * MASK_WARPS;
+      if (w >= words) break;
+      const uint32_t bits = __ballot_sync(0xffffffffu, u[q] && t0 + w * 32 + lane < t1);
+      if (lane < MASK_CTAS) st_peer(peer_shared(&s_bits[t0 / 32 + w], lane), bits);
+    }
   }
-  uni[i] = u;
-}
-
-// Pass 3: (2r+1)^2 dilation on the grid, and the per-CTA dirty count.
-__global__ void __launch_bounds__(MASK_ROWS)
-mask_dilate_kernel(const uint8_t* __restrict__ uni, int gh, int gw, int r,
-                   uint8_t* __restrict__ mask, int* __restrict__ cnt) {
-  pdl_wait();
-  pdl_trigger();
-  const int N = gh * gw;
-  const int i = blockIdx.x * MASK_ROWS + threadIdx.x;
-  int m = 0;
-  if (i < N) {
-    const int y = i / gw, x = i - (i / gw) * gw;
-    const int y0 = max(0, y - r), y1 = min(gh - 1, y + r);
-    const int x0 = max(0, x - r), x1 = min(gw - 1, x + r);
-    for (int yy = y0; yy <= y1 && !m; ++yy)
-      for (int xx = x0; xx <= x1; ++xx)
-        if (uni[yy * gw + xx]) { m = 1; break; }
-    mask[i] = uint8_t(m);
+  cluster_barrier();
+  // dilation: any union token among the row's tokens x - r .. x + r of the
+  // rows y - r .. y + r (at most 17 consecutive bits a row, in two words)
+  const int nw = (N + 31) / 32;
+  uint32_t mine[MASK_WPW];  // this warp's mask words
+#pragma unroll
+  for (int q = 0; q < MASK_WPW; ++q) {
+    const int w = warp + q * MASK_WARPS, i = t0 + w * 32 + lane;
+    bool m = false;
+    if (w < words && i < t1) {
+      const int y = i / gw, x = i - y * gw;
+      const int x0 = max(0, x - r), len = min(gw - 1, x + r) - x0 + 1;
+      const int y1 = min(gh - 1, y + r);
+      for (int yy = max(0, y - r); yy <= y1; ++yy) {
+        const int p = yy * gw + x0, k = p >> 5;
+        const uint32_t win =
+            __funnelshift_r(s_bits[k], k + 1 < nw ? s_bits[k + 1] : 0u, p & 31);
+        m |= (win & ((1u << len) - 1u)) != 0u;
+      }
+      mask[i] = uint8_t(m);
+    }
+    mine[q] = __ballot_sync(0xffffffffu, m);
+    if (w < words && lane == 0) s_word[w] = __popc(mine[q]);
   }
-  int c = __syncthreads_count(m);
-  if (threadIdx.x == 0) cnt[blockIdx.x] = c;
-}
-
-// Pass 4: compaction.  Each CTA sums the counts of the CTAs before it, then a
-// warp ballot + prefix over warps gives each dirty token its slot; the
-// indices come out in ascending token order.
-__global__ void __launch_bounds__(MASK_ROWS)
-mask_compact_kernel(const uint8_t* __restrict__ mask, const int* __restrict__ cnt, int N,
-                    int32_t* __restrict__ idx, int32_t* __restrict__ count) {
-  pdl_wait();
-  pdl_trigger();
-  __shared__ int s_warp[MASK_ROWS / 32];
-  __shared__ int s_base;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x < 32) {
-    int acc = 0;
-    for (int b = lane; b < int(blockIdx.x); b += 32) acc += cnt[b];
-    acc = __reduce_add_sync(0xffffffffu, acc);
-    if (lane == 0) s_base = acc;
-  }
-  const int i = blockIdx.x * MASK_ROWS + threadIdx.x;
-  const int m = (i < N) ? mask[i] : 0;
-  const unsigned bal = __ballot_sync(0xffffffffu, m);
-  if (lane == 0) s_warp[warp] = __popc(bal);
   __syncthreads();
-  int before = s_base;
-  for (int w = 0; w < warp; ++w) before += s_warp[w];
-  if (m) idx[before + __popc(bal & ((1u << lane) - 1u))] = i;
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-    int total = s_base;
-    for (int w = 0; w < MASK_ROWS / 32; ++w) total += s_warp[w];
-    *count = total;
+  // tokens before each of the CTA's words, and the CTA's count to every CTA
+  if (warp == 0) {
+    int base = 0;
+    for (int w0 = 0; w0 < words; w0 += 32) {
+      const int c = w0 + lane < words ? s_word[w0 + lane] : 0;
+      int inc = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      if (w0 + lane < words) s_word[w0 + lane] = base + inc - c;
+      base += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    if (lane < MASK_CTAS) st_peer(peer_shared(&s_cnt[rank], lane), uint32_t(base));
   }
+  cluster_barrier();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int c = 0; c < MASK_CTAS; ++c) {
+    before += c < rank ? s_cnt[c] : 0;
+    total += s_cnt[c];
+  }
+#pragma unroll
+  for (int q = 0; q < MASK_WPW; ++q) {
+    const int w = warp + q * MASK_WARPS;
+    if (w < words && (mine[q] >> lane) & 1u)
+      idx[before + s_word[w] + __popc(mine[q] & ((1u << lane) - 1u))] = t0 + w * 32 + lane;
+  }
+  if (rank == 0 && threadIdx.x == 0) *count = total;
 }
+
+// The cluster reads the map itself up to this many scores (tokens x delta
+// tokens x slices).  Measured, one launch / two: 768 scores 4.7 / 5.2 us, 5120
+// 5.9 / 6.4, 16384 6.8 / 6.5, 32768 (4096 tokens) 9.4 / 8.1: eight SMs fetch
+// the scattered sectors of a larger map too slowly.
+constexpr long long MASK_CLUSTER_SCORES = 8192;
 
 cudaError_t launch_localize(const float* A, int S, int N, int M, int gh, int gw,
                             const DeltaIds& ids, float tau, int dilation, uint8_t* mask,
                             int32_t* idx, int32_t* count, void* ws, cudaStream_t st) {
+  if (N > MASK_MAX_TOKENS) return cudaErrorInvalidValue;
   const int nblk = cdiv(N, MASK_ROWS);
   MaskWs w = carve(ws, N, ids.n);
-  RC_TRY(launch_k(mask_colstats_kernel, dim3(nblk), dim3(MASK_ROWS), 0, st, A, S, N, M, ids,
-                  w.abar, w.part));
-  RC_TRY(launch_k(mask_threshold_kernel, dim3(nblk), dim3(MASK_ROWS), 0, st, w.abar, w.part, nblk,
-                  N, ids, tau, w.uni));
-  RC_TRY(launch_k(mask_dilate_kernel, dim3(nblk), dim3(MASK_ROWS), 0, st, w.uni, gh, gw, dilation,
-                  mask, w.cnt));
-  RC_TRY(launch_k(mask_compact_kernel, dim3(nblk), dim3(MASK_ROWS), 0, st, mask, w.cnt, N, idx,
-                  count));
-  count_launches(4);
+  const bool from_map = 1ll * N * ids.n * S <= MASK_CLUSTER_SCORES;
+  if (!from_map)
+    RC_TRY(launch_k(mask_colstats_kernel, dim3(nblk, ids.n), dim3(MASK_ROWS), 0, st, A, S, N, M,
+                    ids, w.abar, w.part));
+  RC_TRY(launch_k_cluster(from_map ? mask_cluster_kernel<true> : mask_cluster_kernel<false>,
+                          dim3(MASK_CTAS), dim3(MASK_THREADS), 0, MASK_CTAS, st, A, S, N, M, gh,
+                          gw, ids, tau, dilation, nblk, w.abar, w.part, mask, idx, count));
+  count_launches(from_map ? 1 : 2);
   return cudaSuccess;
 }
 
