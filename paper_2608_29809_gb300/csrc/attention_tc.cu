@@ -4,32 +4,42 @@
 // whose dirty rows the QKV GEMM has just refreshed; in the text cross-
 // attention they are the per-layer text keys / values.
 //
-// One work unit = 128 queries of one head over one split of the keys.  CTAs
-// are persistent and warp-specialised:
-//   warp 0     TMA: Q once per unit, then K/V blocks of 64 keys (4 stages).
-//              Every operand comes through 3-D tensor maps (head_dim, head,
-//              row) as a 64-wide 128B-swizzled tile plus a 16-wide 32B-
-//              swizzled tail; the head_dim extent is the true 72, so the pad
-//              to 80 reads as zero and adds nothing to Q K^T.
-//   warp 1     TMEM owner and MMA issuer, polling its inputs: O += P V
-//              (M=128, N=80, 4 K-steps of 16 keys; P read from TMEM as the A
-//              operand, V from shared memory as an MN-major B operand) as
-//              soon as P is ready, and S = Q K^T (M=128, N=64, 5 K-steps of
-//              16) into one of two TMEM S buffers as soon as the block's K/V
-//              have landed and the softmax has read that buffer's last S
-//              (so S runs up to two blocks ahead of the softmax).
-//   warps 2-5  softmax, one thread per query row: reads its S row from TMEM
-//              (freeing the buffer), online softmax in base 2 with lazy
-//              rescaling (O in TMEM is rescaled only when the running max
-//              grows by more than 2^8), and writes its P row (bf16 pairs) to
-//              the TMEM P buffer once the previous P V has read it.  At the
-//              end it normalises O.
-// Two CTAs share an SM (256 TMEM columns and ~100 KB of shared memory each),
-// so the softmax of one overlaps the MMAs and exponentials of the other.
-// Key splits of the same (query tile, head) leave their unnormalised O and
-// row max / sum in a workspace (as column planes, so that the softmax
-// threads' stores are whole 512-byte runs); a small combine kernel, launched
-// right after, merges them (one lane per row).
+// One work unit = one or two tiles of 128 queries of one head over the keys
+// (or a share of them), in blocks of 80 keys; one persistent CTA per SM.  Two
+// streams, each with its own S / P and O in tensor memory, its own issuing
+// warp and its own four softmax warps, share every K and V block (two tiles:
+// a stream each) or take the blocks in turn (one tile; their results are
+// merged when the unit ends).
+//   warp 0        Q and K: TMA, and cp.async for the last 8 head dims
+//   warps 1, 3    a stream's S = Q K^T (M = 128, N = 80, 5 K-steps of 16) and
+//                 O += P V (M = 128, N = 80, 5 K-steps of 16 keys; P read from
+//                 TMEM as the A operand, V from shared memory, MN-major);
+//                 warp 1 owns the tensor memory
+//   warp 2        V, as K
+//   warps 4-7     softmax of stream 0, one thread per query row
+//   warps 8-11    softmax of stream 1
+// Operands come through 3-D tensor maps (head_dim, head, row) as a 64-wide
+// 128B-swizzled tile plus a tail; the head_dim extent is the true 72, and the
+// pad to 80 is zero and adds nothing to Q K^T.  A stream's S has two buffers,
+// and its P replaces the S that it came from, so that S of the next block is
+// there when the softmax of this one ends.  The softmax (base 2) takes a max
+// in a stream's first block only: later blocks use the same reference unless
+// their exponentials grow past 2^64 of it (then the reference is raised, O
+// rescaled and the block done again).
+//
+// What bounds it (80 keys, both streams): the tensor pipe and the shared
+// memory that feeds it 1180 cycles without any softmax (920 of MMA, the rest
+// TMA writes), the softmax 1250 without any MMA (640 of exponentials at 32 per
+// cycle and SM; two warps a scheduler), together 1430.  Measured, earlier form
+// (two CTAs an SM, 64-key blocks, one tile each, K and V tails through TMA,
+// a max per block) -> this one: 831 x 4096 (with the combine kernel it needed)
+// 36.4 -> 27.4 us, 4096 x 4096 116.6 -> 82.9, 3248 x 16384 326 -> 229 (1.07
+// PFLOP/s), 132 x 1024 13.7 -> 10.3.
+//
+// Pairs left over by the last whole wave can have their keys shared by up to
+// nine units.  Each leaves its unnormalised O with the rows' reference and sum
+// in a workspace (as column planes, so that accesses are whole 512-byte runs),
+// and the CTA that finishes last merges them.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <math.h>
@@ -47,15 +57,19 @@ namespace {
 
 using namespace rc::tc;
 
-constexpr int BQ = 128, BKV = 64, THREADS = 192;
-constexpr int TMEM_COLS = 256;     // S0 | S1 (64 columns each) | O (80) | P (32)
-constexpr int CTAS_PER_SM = 2;
+constexpr int BQ = 128, BKV = 80, THREADS = 384;
+// TMEM columns: two S buffers of each stream (P goes over the first half of
+// its S), then O (80 each)
+constexpr int TMEM_COLS = 512;
+constexpr uint32_t TM_O = 4 * BKV, TM_O_STEP = 80;
+static_assert(TM_O + 2 * TM_O_STEP <= TMEM_COLS, "two streams fit the tensor memory");
+__device__ __forceinline__ uint32_t tm_s(int x, int b) { return uint32_t(BKV * (2 * x + b)); }
 // floats per row of a workspace slot: a piece's DH columns, its row max and
-// sum (stored as column planes, see attn_combine_kernel)
+// sum (as column planes: DH / 4 planes of 128 float4, then 128 (max, sum))
 constexpr int PART_STRIDE = 76;
 static_assert(72 + 2 <= PART_STRIDE, "a slot holds DH + 2 floats per row");
-constexpr float LAZY_RESCALE = 8.f;
-constexpr int MIN_KB_PER_SPLIT = 4;  // key blocks per CTA range, at least
+// A block's sum of exponentials past which its reference is raised.
+constexpr float RAISE_SUM = 18446744073709551616.f;  // 2^64
 
 // Packed f32x2 arithmetic (two lanes of f32 per 64-bit register pair).
 __device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
@@ -77,6 +91,35 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
   return d;
 }
 
+// The softmax's steps on columns in registers, in the order they are written.
+__device__ __forceinline__ void scale_pair(uint32_t& a, uint32_t& b, uint64_t scale,
+                                           uint64_t shift) {
+  asm volatile(
+      "{\n\t.reg .b64 t;\n\tmov.b64 t, {%0, %1};\n\t"
+      "fma.rn.f32x2 t, t, %2, %3;\n\tmov.b64 {%0, %1}, t;\n\t}"
+      : "+r"(a), "+r"(b)
+      : "l"(scale), "l"(shift));
+}
+__device__ __forceinline__ void exp_in_place(uint32_t& a) {
+  asm volatile("ex2.approx.ftz.f32 %0, %0;" : "+r"(a));
+}
+__device__ __forceinline__ void sum_pair(uint64_t& s, uint32_t a, uint32_t b) {
+  asm volatile("{\n\t.reg .b64 t;\n\tmov.b64 t, {%1, %2};\n\tadd.rn.f32x2 %0, %0, t;\n\t}"
+               : "+l"(s)
+               : "r"(a), "r"(b));
+}
+__device__ __forceinline__ uint32_t pack_pair(uint32_t lo, uint32_t hi) {
+  uint32_t d;
+  asm volatile("cvt.rn.bf16x2.f32 %0, %2, %1;"
+               : "=r"(d)
+               : "f"(__uint_as_float(lo)), "f"(__uint_as_float(hi)));
+  return d;
+}
+
+// The reference a row's exponents are taken against: its max, or 0 when every
+// score so far is -inf (whose exponentials are then 0, not NaN).
+__device__ __forceinline__ float finite_max(float m) { return m == -INFINITY ? 0.f : m; }
+
 template <int DH>
 struct ACfg {
   static_assert(DH == 64 || DH == 72, "head_dim 64 or 72");
@@ -88,16 +131,22 @@ struct ACfg {
   static constexpr int K128 = BKV * 128, K32 = TAIL ? BKV * 32 : 0;
   // K: 64-wide SW128 tile + 16-wide SW32 tail (the S MMA reads them as two
   // K-major operands); V: one SW128 atom per 64 head-dim columns, so that P V
-  // is a single MMA of N = DHP per 16 keys (MN-major B spanning the atoms)
-  static constexpr int K_BYTES = K128 + K32;
-  static constexpr int V_BYTES = TAIL ? 2 * K128 : K128;
-  // separate rings: K (read by the S MMAs, refilled by the thread that
-  // issues them) and V (read by the P V MMAs, refilled by their issuer)
-  static constexpr int K_STAGES = TAIL ? 4 : 5;
-  static constexpr int V_STAGES = TAIL ? 3 : 4;
+  // is a single MMA of N = DHP per 16 keys (MN-major B spanning the atoms).
+  // Of the second atom only 32 bytes a row are used, so four stages share one
+  static constexpr int K_STAGES = 6;
+  static constexpr int V_STAGES = 7;
   static constexpr int Q_BYTES = Q128 + Q32;
-  static constexpr size_t SMEM =
-      size_t(Q_BYTES) + K_STAGES * K_BYTES + V_STAGES * V_BYTES + 1024 + 256;
+  static constexpr int K_STRIDE = (K128 + K32 + 1023) & ~1023;  // bytes between K stages
+  static constexpr int V_TAILS = TAIL ? (V_STAGES + 3) / 4 : 0;
+  static constexpr size_t SMEM = size_t(2) * Q_BYTES + K_STAGES * K_STRIDE +
+                                 size_t(V_STAGES + V_TAILS) * K128 + 1024;
+  static_assert(Q_BYTES % 1024 == 0 && K128 % 1024 == 0, "128B-swizzled tiles start on 1024 bytes");
+  // byte offset of V stage s and of its tail (32 s mod 128 into the rows of
+  // a shared atom) from the start of the V ring
+  __host__ __device__ static constexpr int v_main(int s) { return s * K128; }
+  __host__ __device__ static constexpr int v_tails(int s) {
+    return (V_STAGES + (s >> 2)) * K128 + 32 * (s & 3);
+  }
   // kind::f16, D f32, A/B bf16; S: both K-major; PV: B (V) MN-major (bit 16)
   static constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) |
                                       (uint32_t(BKV >> 3) << 17) | (uint32_t(BQ >> 4) << 24);
@@ -123,166 +172,222 @@ __device__ __forceinline__ int query_tiles(const RowMap& rm, int n_items, int D)
   return rm.meta ? __ldg(rm.meta + META_TILE + n_items) : (D + BQ - 1) / BQ;
 }
 
-// Work list of one launch, identical in every thread.  A pair = one query
-// tile of one head (heads outermost).  With at least 2 MIN_KB_PER_SPLIT key
-// blocks (the self-attention) the (pair, key block) sequence is cut into G
-// equal contiguous ranges, one per CTA (stream-K): every CTA does the same
-// number of key blocks, and a pair cut by a range boundary leaves partial
-// results (unnormalised O, row max and sum) that the combine kernel merges.
-// With fewer key blocks (the text cross-attention) every pair is one unit,
-// handed out round-robin.
+// A query group: one tile of 128 rows of an item, or two.  A pair = one query
+// group of one head (heads outermost).  Whole waves of pairs are one unit
+// each; the R pairs left over may have their keys shared by `split` units
+// each, in one wave.
 //
-// G: as many CTAs as the grid holds (at least MIN_KB_PER_SPLIT key blocks
-// each), unless ranges of r key blocks, r a power of two dividing the pair's
-// count, cost less: then every CTA holds exactly one piece of one pair.  The
-// estimate is the busiest CTA's key blocks plus PIECE_COST per piece it
-// holds (a piece costs a Q load, a drained O and a stored partial; the equal
-// cut leaves most CTAs two).  Measured on the 4096-token step: at 205 dirty
-// queries (2048 key blocks) 304 ranges of 6-7 blocks gave 441 steps/s, 256
-// of 8 blocks 460; at 410 (4096 key blocks) 304 of 13-14 gave 363, 256 of 16
-// gave 389; from 831 queries on, the equal cut stays.
-struct AttnSched {
-  int qtiles, pairs, nkb, G, total;
-  bool streamk;
-  static constexpr int PIECE_COST = 4;  // key blocks
-  __device__ void init(int tiles, int heads, int Nk, int grid) {
-    qtiles = tiles;
-    pairs = qtiles * heads;
+// The plan of a launch, tabulated by the host for 1 .. PLAN_TABLE query groups
+// of one and of two tiles: the estimated duration and the split that gives it.
+// The device picks the cheaper (a batch's items fill their groups unevenly,
+// and only it knows their counts); larger launches take two tiles and no split.
+constexpr int PLAN_TABLE = 160, MAX_SPLIT = 9;
+struct PlanTable {
+  uint16_t cost[2][PLAN_TABLE];
+  uint8_t split[2][PLAN_TABLE];  // 0: not tabulated
+};
+// Estimated duration in units of 10 ns, fitted to launches of 39 .. 4096
+// queries over 131 .. 16384 keys with every split: a block of 80 keys takes
+// 0.45 us for one tile and 0.74 us for two, a wave UNIT more, and the merge of
+// shared pairs, by the last of their units, MERGE + MERGE_SHARE per share.
+// (4096 keys, the best / the next plan in us: 201 queries one tile split in
+// four 15.3 / two tiles 21.2; 831 one tile whole 27.4 / two tiles split in two
+// 30.2; 4096 two tiles whole 82.9 / one tile 94.6; 3248 queries over 16384
+// keys two tiles, the rest split in two 229 / whole 291.)
+constexpr int BLOCK1 = 45, BLOCK2 = 74, UNIT = 60;
+constexpr int MERGE1 = 400, MERGE2 = 480, MERGE_SHARE1 = 30, MERGE_SHARE2 = 90;
+constexpr int SLOTS_PER_SM = 2;    // workspace slots: two tiles of a shared unit
+constexpr int CAPTURE_KEYS = 448;  // keys of a launch that captures probabilities, at most
+int plan_cost(int pairs, int nkb, int grid, int tiles, int split) {
+  const int block = tiles == 2 ? BLOCK2 : BLOCK1;
+  if (split == 1) return (pairs + grid - 1) / grid * (nkb * block + UNIT);
+  return pairs / grid * (nkb * block + UNIT) + (nkb + split - 1) / split * block + UNIT +
+         (tiles == 2 ? MERGE2 + MERGE_SHARE2 * split : MERGE1 + MERGE_SHARE1 * split);
+}
+int pick_split(int pairs, int nkb, int grid, int tiles, int* cost) {
+  int best = 1;
+  *cost = plan_cost(pairs, nkb, grid, tiles, 1);
+  const int rest = pairs % grid;
+  for (int s = 2; s <= MAX_SPLIT && s <= nkb && rest > 0 && rest * s <= grid; ++s) {
+    const int c = plan_cost(pairs, nkb, grid, tiles, s);
+    if (c < *cost) {
+      *cost = c;
+      best = s;
+    }
+  }
+  return best;
+}
+
+__device__ __forceinline__ int query_groups(const RowMap& rm, int n_items, int D, int rows) {
+  if (!rm.meta) return (D + rows - 1) / rows;
+  int g = 0;
+  for (int i = 0; i < n_items; ++i) g += (__ldg(rm.meta + META_CNT + i) + rows - 1) / rows;
+  return g;
+}
+__device__ __forceinline__ TileLoc locate_group(const RowMap& rm, int n_items, int D, int rows,
+                                                int g) {
+  if (!rm.meta) return TileLoc{0, g * rows, min(rows, D - g * rows)};
+  int i = 0, c = __ldg(rm.meta + META_CNT);
+  while (i + 1 < n_items && g >= (c + rows - 1) / rows) {
+    g -= (c + rows - 1) / rows;
+    c = __ldg(rm.meta + META_CNT + ++i);
+  }
+  return TileLoc{i, __ldg(rm.meta + META_OFF + i) + g * rows, min(rows, c - g * rows)};
+}
+
+// The units of one CTA, handed out round robin.
+struct AttnUnits {
+  int groups, rows, split, whole, units, nkb;
+  __device__ void init(const PlanTable& pt, const RowMap& rm, int n_items, int D, int heads, int Nk,
+                       int grid) {
     nkb = (Nk + BKV - 1) / BKV;
-    total = pairs * nkb;
-    streamk = nkb >= 2 * MIN_KB_PER_SPLIT;
-    G = grid;
-    if (!streamk) return;
-    G = pick_ctas(total, nkb, grid);
+    const int tiles = query_tiles(rm, n_items, D);
+    rows = 2 * BQ;
+    split = 1;
+    groups = query_groups(rm, n_items, D, rows);
+    if (tiles >= 1 && tiles <= PLAN_TABLE && pt.split[0][0]) {
+      const bool one = pt.cost[0][tiles - 1] < pt.cost[1][groups - 1];
+      split = one ? pt.split[0][tiles - 1] : pt.split[1][groups - 1];
+      if (one) {
+        rows = BQ;
+        groups = tiles;
+      }
+    }
+    const int pairs = groups * heads;
+    whole = split == 1 ? pairs : pairs / grid * grid;
+    units = whole + (pairs - whole) * split;
   }
-  // (powers of two only, found with shifts: every thread of the attention
-  // and combine kernels runs this before its first load, and a search with
-  // run-time divisors cost more than the better ranges saved; not inlined,
-  // so that its temporaries do not raise the kernels' register counts)
-  static __device__ __noinline__ int pick_ctas(int total, int nkb, int grid) {
-    const int G = max(1, min(grid, total / MIN_KB_PER_SPLIT));
-    if (nkb & (nkb - 1)) return G;
-    int lg = 0;
-    while ((1 << lg) < MIN_KB_PER_SPLIT) ++lg;
-    while ((1 << lg) < nkb && (total >> lg) > grid) ++lg;
-    if ((1 << lg) > nkb || (total >> lg) > grid) return G;
-    const int r0 = (total + G - 1) / G;
-    const bool one_piece = total % G == 0 && nkb % r0 == 0;
-    return (1 << lg) + PIECE_COST < r0 + PIECE_COST * (one_piece ? 1 : 2) ? total >> lg : G;
-  }
-  // unsigned 32-bit arithmetic: the launcher checks total * G < 2^32
-  __device__ int bound(int c) const { return int(unsigned(total) * unsigned(c) / unsigned(G)); }
-  // the CTA whose range holds key-block position pos (0 <= pos < total)
-  __device__ int cta_of(int pos) const {
-    int c = int(unsigned(pos) * unsigned(G) / unsigned(total));
-    while (c > 0 && bound(c) > pos) --c;
-    while (c + 1 < G && bound(c + 1) <= pos) ++c;
-    return c;
+};
+struct AttnUnit {
+  int pair, g, h, kb0, kb1;
+  int share;  // index among the shared units, -1 for a whole pair
+  __device__ void set(const AttnUnits& un, int u) {
+    int q = 0, n = 1;
+    pair = u;
+    share = -1;
+    if (u >= un.whole) {
+      share = u - un.whole;
+      n = un.split;
+      pair = un.whole + share / n;
+      q = share - share / n * n;
+    }
+    h = pair / un.groups;
+    g = pair - h * un.groups;
+    kb0 = un.nkb * q / n;
+    kb1 = un.nkb * (q + 1) / n;
   }
 };
 
-// One CTA's segments in order: (pair, key blocks [kb0, kb1), slot), slot -1
-// for a whole pair (its normalised output is written directly), 0 / 1 for
-// the CTA's first / last partial piece (workspace slot 2 c + slot).
-struct AttnSeg {
-  const AttnSched* sc;
-  int cur, end;
-  bool first;
-  __device__ void init(const AttnSched& s, int c) {
-    sc = &s;
-    first = true;
-    if (s.streamk) {
-      cur = c < s.G ? s.bound(c) : 0;
-      end = c < s.G ? s.bound(c + 1) : 0;
-    } else {
-      cur = c;  // next pair
-      end = s.pairs;
+// The last 8 of 72 head dims of a key block: 16 bytes a row, through cp.async
+// (a TMA box takes as long for a row of 16 bytes as for one of 128: with
+// 16-wide boxes for the tails 112 rows of K and V took 1043 cycles to load,
+// with a 64-wide one for V 1210, without them 610).  Byte offset of 16-byte chunk j
+// of row r in the K tail (32-byte rows, 32B swizzle) and in V's second atoms
+// (128-byte rows, 128B swizzle; stage s has chunks 2 (s mod 4) and the next).
+__device__ __forceinline__ int k_tail(int r, int j) { return r * 32 + 16 * (j ^ ((r >> 2) & 1)); }
+__device__ __forceinline__ int v_tail(int r, int j) { return r * 128 + 16 * (j ^ (r & 7)); }
+template <bool V>
+__device__ __forceinline__ void load_tail(uint8_t* dst, int chunk, const bf16* src, int ld,
+                                          int row0, int rows, int lane) {
+#pragma unroll
+  for (int q = 0; q < (BKV + 31) / 32; ++q) {
+    const int r = q * 32 + lane;
+    if (r < BKV) {
+      // rows past the end are filled with zeros, as the TMA does
+      const bool in = row0 + r < rows;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                       saddr(dst + (V ? v_tail(r, chunk) : k_tail(r, chunk)))),
+                   "l"(src + size_t(in ? row0 + r : 0) * ld), "r"(in ? 16 : 0)
+                   : "memory");
     }
   }
-  __device__ bool next(int& pair, int& kb0, int& kb1, int& slot) {
-    if (cur >= end) return false;
-    if (!sc->streamk) {
-      pair = cur;
-      kb0 = 0;
-      kb1 = sc->nkb;
-      slot = -1;
-      cur += sc->G;
-      return true;
-    }
-    pair = cur / sc->nkb;
-    kb0 = cur - pair * sc->nkb;
-    kb1 = min(sc->nkb, kb0 + (end - cur));
-    cur += kb1 - kb0;
-    slot = (kb0 == 0 && kb1 == sc->nkb) ? -1 : (first ? 0 : 1);
-    first = false;
-    return true;
-  }
-};
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+// The tails of all but the last PENDING of the blocks issued so far (g) have
+// landed: made visible to the tensor core, and their stages' barriers told
+// (told counts the blocks).
+template <int PENDING>
+__device__ __forceinline__ void tell_tails(int g, int& told, uint32_t full, int stages, int lane) {
+  asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+  if (told >= g - PENDING) return;
+  fence_proxy_async_smem();
+  __syncwarp();
+  for (; told < g - PENDING; ++told)
+    if (lane == 0) mbar_arrive(full + 8 * (told % stages));
+}
 
-template <int DH>
-__global__ void __launch_bounds__(THREADS, CTAS_PER_SM)
+template <int DH, bool CAP>
+__global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmQt,
-               const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmKt,
-               const __grid_constant__ CUtensorMap tmV, const __grid_constant__ AttnItems ai, int Nk, bf16* __restrict__ O, int ldo,
+               const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+               const bf16* __restrict__ Kp, const bf16* __restrict__ Vp, int ldkv, int kv_rows,
+               const __grid_constant__ AttnItems ai, const __grid_constant__ PlanTable pt,
+               int Nk, bf16* __restrict__ O, int ldo,
                int heads, RowMap rm, float scale_log2, unsigned* err, float* __restrict__ part,
-               const __grid_constant__ AttnCapture cap) {
+               unsigned* __restrict__ ticket, const __grid_constant__ AttnCapture cap) {
   using C = ACfg<DH>;
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~uintptr_t(1023));
   constexpr int KS = C::K_STAGES, VS = C::V_STAGES;
-  uint8_t* sQ = smem;
-  uint8_t* sK = sQ + C::Q_BYTES;
-  uint8_t* sV = sK + KS * C::K_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sV + VS * C::V_BYTES);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 30);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  // barrier addresses
-  const uint32_t b0 = saddr(bars);
-  const uint32_t q_full = b0, q_empty = b0 + 8;
-  const uint32_t k_full = b0 + 16, k_empty = k_full + 8 * KS;
-  const uint32_t v_full = k_empty + 8 * KS;
-  const uint32_t s_full = v_full + 8 * VS;           // [2]: S of a block is in TMEM
-  const uint32_t s_free = s_full + 16;               // [2]: the softmax has read it
-  const uint32_t p_ready = s_free + 16;              // P of the next block is in TMEM
-  const uint32_t pv_done = p_ready + 8;              // one phase per completed P V
-  const uint32_t o_full = pv_done + 8, o_free = o_full + 8;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* sQ = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                           ~uintptr_t(1023));
+  uint8_t* sK = sQ + 2 * C::Q_BYTES;
+  uint8_t* sV = sK + KS * C::K_STRIDE;
+  constexpr int BARS = 2 + 2 * KS + 2 * VS + 12 + 3;
+  __shared__ uint64_t bars[BARS];
+  __shared__ float2 s_ml[2][2][BQ];  // (max, sum) of the streams' rows, units alternating
+  __shared__ uint32_t tmem_slot;
+  __shared__ int s_abort, s_last;
+  volatile int* abort_flag = &s_abort;
+  const uint32_t q_full = saddr(bars), q_empty = q_full + 8;
+  const uint32_t k_full = q_empty + 8, k_empty = k_full + 8 * KS;          // [KS]
+  const uint32_t v_full = k_empty + 8 * KS, v_empty = v_full + 8 * VS;      // [VS]
+  const uint32_t s_full = v_empty + 8 * VS;                                 // [stream][buffer]
+  const uint32_t p_ready = s_full + 32, pv_done = p_ready + 32;             // [stream][buffer]
+  const uint32_t o_full = pv_done + 32, o_free = o_full + 8;
+  const uint32_t meet = o_free + 8;  // the softmax warps of both streams
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    mbar_init(q_full, 1);
-    mbar_init(q_empty, 1);
-    for (int s = 0; s < KS; ++s) {
-      mbar_init(k_full + 8 * s, 1);
-      mbar_init(k_empty + 8 * s, 1);
+    for (int i = 0; i < BARS; ++i) mbar_init(q_full + 8 * i, 1);
+    for (int i = 0; i < KS; ++i) mbar_init(k_empty + 8 * i, 2);
+    for (int i = 0; i < VS; ++i) mbar_init(v_empty + 8 * i, 2);
+    mbar_init(q_empty, 2);
+    mbar_init(o_full, 2);
+    if (C::TAIL) {  // the TMA's arrival and that of the tail's warp
+      for (int i = 0; i < KS; ++i) mbar_init(k_full + 8 * i, 2);
+      for (int i = 0; i < VS; ++i) mbar_init(v_full + 8 * i, 2);
     }
-    for (int s = 0; s < VS; ++s) mbar_init(v_full + 8 * s, 1);
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(s_full + 8 * b, 1);
-      mbar_init(s_free + 8 * b, 128);
-    }
-    mbar_init(p_ready, 128);
-    mbar_init(pv_done, 1);
-    mbar_init(o_full, 1);
-    mbar_init(o_free, 128);
-    *abort_flag = 0;
+    for (int i = 0; i < 4; ++i) mbar_init(p_ready + 8 * i, 4);
+    mbar_init(o_free, 8);
+    mbar_init(meet, 8);
+    s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(saddr(tmem_slot), TMEM_COLS);
-  if (warp == 0 && lane == 0) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmQ)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
-    if (C::TAIL) {
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmQt)) : "memory");
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmKt)) : "memory");
+  if (warp == 1) tmem_alloc(saddr(&tmem_slot), TMEM_COLS);
+  if (warp == 0 && elect_one()) {
+    const CUtensorMap* maps[4] = {&tmQ, &tmK, &tmV, &tmQt};
+#pragma unroll
+    for (int i = 0; i < (C::TAIL ? 4 : 3); ++i)
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(maps[i])) : "memory");
+  }
+  if (C::TAIL) {
+    // head dims 72 .. 79 of every K and V stage: zero, and never written again
+    const uint4 z = make_uint4(0, 0, 0, 0);
+    for (int i = threadIdx.x; i < KS * BKV; i += THREADS) {
+      const int r = i % BKV;
+      *reinterpret_cast<uint4*>(sK + (i / BKV) * C::K_STRIDE + C::K128 + k_tail(r, 1)) = z;
     }
+    for (int i = threadIdx.x; i < VS * BKV; i += THREADS) {
+      const int r = i % BKV;
+      const int s = i / BKV;
+      *reinterpret_cast<uint4*>(sV + C::v_tails(s & ~3) + v_tail(r, 2 * (s & 3) + 1)) = z;
+    }
+    fence_proxy_async_smem();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-  const uint32_t tS0 = tmem_base, tO = tmem_base + 2 * BKV, tP = tO + 80;
+  const uint32_t tmem = tmem_slot;
 
   // the live row count (and, for several items, the row table) was written
   // two or more launches earlier: read before the programmatic-dependency
@@ -290,317 +395,394 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   // letting its successor start); Q and the fresh K / V rows come from the
   // predecessor
   const int D = live_count(rm.count, rm.bound, err);
-  AttnSched sc;
-  sc.init(query_tiles(rm, ai.n, D), heads, Nk, gridDim.x);
+  AttnUnits un;
+  un.init(pt, rm, ai.n, D, heads, Nk, int(gridDim.x));
+  const int u0 = blockIdx.x, du = gridDim.x;
   pdl_wait();
   pdl_trigger();
 
-  // Two issuing threads, so that neither MMA stream waits behind the other's
-  // instruction issue: warp 0 loads Q and K and issues the S MMAs, warp 1
-  // loads V and issues the P V MMAs.  Each refills its own ring.
   if (warp == 0) {
-    // ------------------------------------------------- Q, K loads and S = Q K^T
-    // K runs KS - 2 key blocks ahead of the S MMAs: the K stage of block
-    // g + KS - 2 is the one block g - 2 used, whose S has long completed, so
-    // the refill never waits on the MMA just issued.  S(g) goes into the S
-    // buffer the softmax of block g - 2 has read.
-    if (lane == 0) {
-      const uint32_t qb = saddr(sQ), kb_0 = saddr(sK);
-      const uint64_t dq = sw128_desc(qb), dqt = sw32_kmajor_desc(qb + C::Q128);
-      // stage descriptors differ only in the start address field (address >>
-      // 4, which never carries out of its 14 bits here)
-      const uint64_t dk = sw128_desc(kb_0), dkt = sw32_kmajor_desc(kb_0 + C::K128);
-      int gl = 0, gs = 0, uc = 0;
-      AttnSeg itl;
-      itl.init(sc, blockIdx.x);
-      int l_kb = 0, l_kb1 = 0, l_h = 0, l_row = 0;
-      bool l_more = true;
-      // requests K of the next key block to load (false: a wait gave up)
-      auto load_k = [&]() -> bool {
-        while (l_kb >= l_kb1) {
-          int pair, kb0, kb1, slot;
-          if (!itl.next(pair, kb0, kb1, slot)) {
-            l_more = false;
-            return true;
-          }
-          const TileLoc tl = locate_tile(rm, ai.n, D, pair % sc.qtiles);
-          l_h = pair / sc.qtiles;
-          l_row = ai.krow[tl.item];
-          l_kb = kb0;
-          l_kb1 = kb1;
-        }
-        const int st = gl % KS;
-        if (!mbar_sleep(k_empty + 8 * st, ((gl / KS) & 1) ^ 1, abort_flag)) return false;
-        mbar_expect_tx(k_full + 8 * st, C::K_BYTES);
-        uint8_t* base = sK + st * C::K_BYTES;
-        tma_load_3d(saddr(base), &tmK, k_full + 8 * st, 0, l_h, l_row + l_kb * BKV);
-        if (C::TAIL)
-          tma_load_3d(saddr(base + C::K128), &tmKt, k_full + 8 * st, 64, l_h, l_row + l_kb * BKV);
-        ++l_kb;
-        ++gl;
-        return true;
-      };
-      AttnSeg it;
-      it.init(sc, blockIdx.x);
-      int pair, kb0, kb1, slot;
-      for (; it.next(pair, kb0, kb1, slot); ++uc) {
-        const int qt = pair % sc.qtiles, h = pair / sc.qtiles;
-        const TileLoc tl = locate_tile(rm, ai.n, D, qt);
-        const int n = kb1 - kb0;
-        // Q of the unit, once the previous unit's S MMAs have read the buffer
-        if (!mbar_sleep(q_empty, (uc + 1) & 1, abort_flag)) goto timeout;
-        mbar_expect_tx(q_full, C::Q_BYTES);
-        tma_load_3d(saddr(sQ), &tmQ, q_full, 0, h, tl.row0);
-        if (C::TAIL) tma_load_3d(saddr(sQ + C::Q128), &tmQt, q_full, 64, h, tl.row0);
-        for (int ns = 0; ns < n; ++ns, ++gs) {
-          while (l_more && gl < gs + KS - 1) {
-            if (!load_k()) goto timeout;
-          }
-          if (ns == 0 && !mbar_sleep(q_full, uc & 1, abort_flag)) goto timeout;
-          const int st = gs % KS;
-          if (!mbar_sleep(k_full + 8 * st, (gs / KS) & 1, abort_flag) ||
-              !mbar_sleep(s_free + 8 * (gs & 1), ((gs >> 1) + 1) & 1, abort_flag))
-            goto timeout;
-          tc_fence_after();
-          const uint64_t so = uint64_t(st * (C::K_BYTES >> 4));
-          const uint32_t sd = tS0 + uint32_t(BKV) * uint32_t(gs & 1);
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            umma_bf16(sd, dq + 2 * kk, dk + so + 2 * kk, C::IDESC_S, kk > 0 ? 1u : 0u);
-          if (C::TAIL) umma_bf16(sd, dqt, dkt + so, C::IDESC_S, 1u);
-          umma_commit(k_empty + 8 * st);
-          umma_commit(s_full + 8 * (gs & 1));
-          if (ns == n - 1) umma_commit(q_empty);  // last S of the unit issued
+    // ------------------------------------------------------------ Q and K
+    const bool leader = elect_one();
+    int g = 0, uc = 0, told = 0;
+    AttnUnit w;
+    for (int u = u0; u < un.units; u += du, ++uc) {
+      w.set(un, u);
+      const TileLoc tl = locate_group(rm, ai.n, D, un.rows, w.g);
+      const int krow = ai.krow[tl.item], tiles = tl.rows > BQ ? 2 : 1;
+      if (!mbar_sleep_warp(q_empty, (uc & 1) ^ 1, abort_flag)) goto timeout;
+      if (leader) {
+        mbar_expect_tx(q_full, tiles * C::Q_BYTES);
+        for (int x = 0; x < tiles; ++x) {
+          uint8_t* q = sQ + x * C::Q_BYTES;
+          tma_load_3d(saddr(q), &tmQ, q_full, 0, w.h, tl.row0 + x * BQ);
+          if (C::TAIL) tma_load_3d(saddr(q + C::Q128), &tmQt, q_full, 64, w.h, tl.row0 + x * BQ);
         }
       }
+      for (int kb = w.kb0; kb < w.kb1; ++kb, ++g) {
+        const int s = g % KS;
+        if (!mbar_sleep_warp(k_empty + 8 * s, ((g / KS) & 1) ^ 1, abort_flag)) goto timeout;
+        uint8_t* b = sK + s * C::K_STRIDE;
+        if (leader) {
+          mbar_expect_tx(k_full + 8 * s, C::K128);
+          tma_load_3d(saddr(b), &tmK, k_full + 8 * s, 0, w.h, krow + kb * BKV);
+        }
+        if (C::TAIL) {
+          load_tail<false>(b + C::K128, 0, Kp + w.h * DH + 64, ldkv, krow + kb * BKV, kv_rows, lane);
+          tell_tails<1>(g + 1, told, k_full, KS, lane);
+        }
+      }
+      // (the next unit's Q waits for this one's last S, which waits for these)
+      if (C::TAIL) tell_tails<0>(g, told, k_full, KS, lane);
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------------ V loads and O += P V
-    // V runs VS key blocks ahead: after P V(g) the thread waits for it to
-    // complete (pv_done, which the softmax waits for too; the thread has time:
-    // P(g + 1) takes a whole softmax) and refills the stage with V(g + VS).
-    if (lane == 0) {
-      const uint64_t dv = sw128_mnmajor_desc_lbo(saddr(sV), C::K128);
-      int gv = 0, g = 0, uc = 0;
-      AttnSeg itl;
-      itl.init(sc, blockIdx.x);
-      int l_kb = 0, l_kb1 = 0, l_h = 0, l_row = 0;
-      bool l_more = true;
-      auto load_v = [&]() -> bool {
-        while (l_kb >= l_kb1) {
-          int pair, kb0, kb1, slot;
-          if (!itl.next(pair, kb0, kb1, slot)) {
-            l_more = false;
-            return true;
+  } else if (warp == 1 || warp == 3) {
+    // ------------------------------------------- S = Q K^T and O += P V of a stream
+    // S runs up to two of the stream's blocks ahead (two buffers); a buffer
+    // takes its next S once the P V of the P in it is done.  A block of a
+    // unit with one tile is one stream's alone, which then frees its K and V
+    // for both
+    if (elect_one()) {
+      const int x = warp >> 1;
+      const uint64_t dq = sw128_desc(saddr(sQ)), dqt = sw32_kmajor_desc(saddr(sQ + C::Q128));
+      const uint64_t dk = sw128_desc(saddr(sK)), dkt = sw32_kmajor_desc(saddr(sK + C::K128));
+      const uint32_t bs = s_full + 16 * x, bp = p_ready + 16 * x, bd = pv_done + 16 * x;
+      const uint32_t to = tmem + TM_O + TM_O_STEP * uint32_t(x);
+      int g0 = 0, uc = 0, ns = 0, np = 0;  // blocks of earlier units; units; S, P V so far
+      AttnUnit w;
+      for (int u = u0; u < un.units; u += du, ++uc) {
+        w.set(un, u);
+        const int n = w.kb1 - w.kb0;
+        const bool two = locate_group(rm, ai.n, D, un.rows, w.g).rows > BQ;
+        const int i0 = two ? 0 : x, di = two ? 1 : 2;
+        const uint64_t qo = two ? uint64_t(x * (C::Q_BYTES >> 4)) : 0;
+        if (!mbar_sleep(q_full, uc & 1, abort_flag)) goto timeout;
+        int is = i0;  // next block to compute S of
+        for (int i = i0; i < n; i += di) {
+          for (; is < n && is < i + 2 * di; is += di, ++ns) {
+            const int g = g0 + is, s = g % KS, b = ns & 1;
+            if (!mbar_sleep(k_full + 8 * s, (g / KS) & 1, abort_flag) ||
+                !mbar_sleep(bd + 8 * b, ((ns >> 1) & 1) ^ 1, abort_flag))
+              goto timeout;
+            tc_fence_after();
+            const uint64_t so = uint64_t(s * (C::K_STRIDE >> 4));
+            const uint32_t sd = tmem + tm_s(x, b);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              umma_bf16(sd, dq + qo + 2 * kk, dk + so + 2 * kk, C::IDESC_S, kk > 0 ? 1u : 0u);
+            if (C::TAIL) umma_bf16(sd, dqt + qo, dkt + so, C::IDESC_S, 1u);
+            umma_commit(bs + 8 * b);
+            umma_commit(k_empty + 8 * s);
+            if (!two) umma_commit(k_empty + 8 * s);
+            if (is + di >= n) umma_commit(q_empty);  // the unit's last S of this stream
           }
-          const TileLoc tl = locate_tile(rm, ai.n, D, pair % sc.qtiles);
-          l_h = pair / sc.qtiles;
-          l_row = ai.vrow[tl.item];
-          l_kb = kb0;
-          l_kb1 = kb1;
-        }
-        const int st = gv % VS;
-        // the stage's previous block, gv - VS, is the P V just issued
-        if (gv >= VS && !mbar_sleep(pv_done, (gv - VS) & 1, abort_flag)) return false;
-        mbar_expect_tx(v_full + 8 * st, C::V_BYTES);
-        uint8_t* base = sV + st * C::V_BYTES;
-        tma_load_3d(saddr(base), &tmV, v_full + 8 * st, 0, l_h, l_row + l_kb * BKV);
-        if (C::TAIL)
-          tma_load_3d(saddr(base + C::K128), &tmV, v_full + 8 * st, 64, l_h, l_row + l_kb * BKV);
-        ++l_kb;
-        ++gv;
-        return true;
-      };
-      while (l_more && gv < VS) {
-        if (!load_v()) goto timeout;
-      }
-      AttnSeg it;
-      it.init(sc, blockIdx.x);
-      int pair, kb0, kb1, slot;
-      for (; it.next(pair, kb0, kb1, slot); ++uc) {
-        const int n = kb1 - kb0;
-        for (int np = 0; np < n; ++np, ++g) {
-          if (np == 0 && !mbar_sleep(o_free, (uc + 1) & 1, abort_flag)) goto timeout;
-          const int st = g % VS;
-          if (!mbar_sleep(p_ready, g & 1, abort_flag) ||
-              !mbar_sleep(v_full + 8 * st, (g / VS) & 1, abort_flag))
+          const int g = g0 + i, s = g % VS, b = np & 1;
+          // O of the previous unit has been read
+          if (i == i0 && !mbar_sleep(o_free, (uc & 1) ^ 1, abort_flag)) goto timeout;
+          if (!mbar_sleep(v_full + 8 * s, (g / VS) & 1, abort_flag) ||
+              !mbar_sleep(bp + 8 * b, (np >> 1) & 1, abort_flag))
             goto timeout;
+          ++np;
           tc_fence_after();
-          const uint64_t vd = dv + uint64_t(st * (C::V_BYTES >> 4));
-          // 16 keys per MMA: P columns 8 kk .., V rows 16 kk .. (2 KB)
+          // keys past the last valid one are left out in steps of 16 (their
+          // values may belong to something else)
+          const int valid = Nk - (w.kb0 + i) * BKV;
+          const uint64_t vd = sw128_mnmajor_desc_lbo(
+              saddr(sV) + uint32_t(C::v_main(s)),
+              C::TAIL ? uint32_t(C::v_tails(s) - C::v_main(s)) : uint32_t(C::K128));
+          const uint32_t tp = tmem + tm_s(x, b);
 #pragma unroll
           for (int kk = 0; kk < BKV / 16; ++kk)
-            umma_bf16_ta(tO, tP + 8 * kk, vd + 128 * kk, C::IDESC_PV,
-                         (np > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(pv_done);
-          if (np == n - 1) umma_commit(o_full);
-          if (l_more && !load_v()) goto timeout;  // V(g + VS) into this stage
+            if (kk == 0 || 16 * kk < valid)
+              umma_bf16_ta(to, tp + 8 * kk, vd + 128 * kk, C::IDESC_PV,
+                           (i > i0 || kk > 0) ? 1u : 0u);
+          umma_commit(bd + 8 * b);
+          umma_commit(v_empty + 8 * s);
+          if (!two) umma_commit(v_empty + 8 * s);
+        }
+        if (i0 >= n) umma_commit(q_empty);  // (no block in this unit)
+        umma_commit(o_full);
+        g0 += n;
+      }
+    }
+  } else if (warp == 2) {
+    // ------------------------------------------------------------ V
+    const bool leader = elect_one();
+    int g = 0, told = 0;
+    AttnUnit w;
+    for (int u = u0; u < un.units; u += du) {
+      w.set(un, u);
+      const int vrow = ai.vrow[locate_group(rm, ai.n, D, un.rows, w.g).item];
+      for (int kb = w.kb0; kb < w.kb1; ++kb, ++g) {
+        const int s = g % VS;
+        if (!mbar_sleep_warp(v_empty + 8 * s, ((g / VS) & 1) ^ 1, abort_flag)) goto timeout;
+        if (leader) {
+          mbar_expect_tx(v_full + 8 * s, C::K128);
+          tma_load_3d(saddr(sV + C::v_main(s)), &tmV, v_full + 8 * s, 0, w.h, vrow + kb * BKV);
+        }
+        if (C::TAIL) {
+          load_tail<true>(sV + C::v_tails(s & ~3), 2 * (s & 3), Vp + w.h * DH + 64, ldkv, vrow + kb * BKV, kv_rows, lane);
+          tell_tails<1>(g + 1, told, v_full, VS, lane);
         }
       }
     }
+    if (C::TAIL) tell_tails<0>(g, told, v_full, VS, lane);
   } else {
     // ------------------------------------------------------------ softmax
-    const int sp4 = warp & 3;
-    const int row = sp4 * 32 + lane;
-    const uint32_t lane_off = uint32_t(sp4 * 32) << 16;
-    int g = 0, uc = 0;
-    AttnSeg it;
-    it.init(sc, blockIdx.x);
-    int pair, kb0, kb1, slot;
-    for (; it.next(pair, kb0, kb1, slot); ++uc) {
-      const int qt = pair % sc.qtiles, h = pair / sc.qtiles;
-      const int n = kb1 - kb0;
+    const int sp = warp & 3, x = (warp - 4) >> 2, row = sp * 32 + lane;
+    const uint32_t lane_off = uint32_t(sp * 32) << 16;
+    const uint32_t to = tmem + TM_O + TM_O_STEP * uint32_t(x) + lane_off;
+    int cnt = 0, uc = 0;  // blocks of this stream, units so far
+    uint32_t met = 0;
+    // one arrival per warp
+    auto arrive = [&](uint32_t bar) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar);
+    };
+    // all eight softmax warps (a bounded wait, like every other)
+    auto join = [&]() {
+      arrive(meet);
+      const bool ok = mbar_sleep_warp(meet, met, abort_flag);
+      met ^= 1;
+      return ok;
+    };
+    AttnUnit w;
+    for (int u = u0; u < un.units; u += du, ++uc) {
+      w.set(un, u);
+      const int n = w.kb1 - w.kb0;
+      const TileLoc tl = locate_group(rm, ai.n, D, un.rows, w.g);
+      const bool two = tl.rows > BQ;
       float m = -INFINITY, l = 0.f;
       float cap_s[8];  // scaled scores of the captured key columns
 #pragma unroll
       for (int q = 0; q < 8; ++q) cap_s[q] = -INFINITY;
-      for (int j = 0; j < n; ++j, ++g) {
-        if (!mbar_sleep_warp(s_full + 8 * (g & 1), (g >> 1) & 1, abort_flag)) goto timeout;
+      for (int i = two ? 0 : x; i < n; i += two ? 1 : 2, ++cnt) {
+        const int b = cnt & 1;
+        const uint32_t ts = tmem + tm_s(x, b) + lane_off;
+        const int key0 = (w.kb0 + i) * BKV, valid = Nk - key0;
+        if (!mbar_sleep_warp(s_full + 8 * (2 * x + b), (cnt >> 1) & 1, abort_flag)) goto timeout;
         tc_fence_after();
+        // p = 2^(s * scale - m) against a reference m (scaled base-2 units;
+        // scale = log2 e / sqrt(dh)), the max of the stream's first block.
+        // The result does not depend on the reference as long as nothing
+        // overflows, so later blocks take no max: only when a block's sum is
+        // past 2^64 (warp-uniform: the TMEM accesses are warp-wide) is the
+        // reference raised and the block, still in its buffer, done again
         uint32_t r[BKV];
+        float bl, alpha = 1.f;
+        // (a row whose scores were all -inf so far has no reference yet)
+        bool take_max = __any_sync(0xffffffffu, m == -INFINITY);
+        for (;;) {
 #pragma unroll
-        for (int i = 0; i < BKV / 16; ++i)
-          tmem_ld16_nowait(tS0 + uint32_t(BKV) * uint32_t(g & 1) + lane_off + 16u * i, r + 16 * i);
-        tmem_wait_ld();
-        if (cap.n) {  // (warp-uniform) the captured columns that fall in this block
+          for (int c = 0; c < BKV / 16; ++c) tmem_ld16_nowait(ts + 16u * c, r + 16 * c);
+          if (CAP) {  // (warp-uniform) the captured columns that fall in this block
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              if (q < cap.n && cap.id[q] >= key0 && cap.id[q] < key0 + BKV)
+                cap_s[q] = __uint_as_float(tmem_ld1_nowait(ts + uint32_t(cap.id[q] - key0)));
+          }
+          tmem_wait_ld();
+          if (valid < BKV) {  // the last, partial key block (warp-uniform)
+#pragma unroll
+            for (int c = 0; c < BKV; ++c)
+              if (c >= valid) r[c] = __float_as_uint(-INFINITY);
+          }
+          if (take_max) {
+            float f8[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f8[q] = __uint_as_float(r[q]);
+#pragma unroll
+            for (int c = 8; c < BKV; ++c) f8[c & 7] = fmaxf(f8[c & 7], __uint_as_float(r[c]));
+            const float mx = fmaxf(fmaxf(fmaxf(f8[0], f8[1]), fmaxf(f8[2], f8[3])),
+                                   fmaxf(fmaxf(f8[4], f8[5]), fmaxf(f8[6], f8[7]))) *
+                             scale_log2;
+            const float mn = fmaxf(m, mx);
+            alpha = m == -INFINITY ? 0.f : ex2_ftz(m - mn);
+            m = mn;
+          }
+          const float mr = finite_max(m);
+          const uint64_t sc2 = f32x2(scale_log2, scale_log2), nm2 = f32x2(-mr, -mr);
+          uint64_t sum2[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) sum2[q] = f32x2(0.f, 0.f);
+          // software-pipelined by hand (the asm statements keep their order):
+          // the scaling runs PIPE columns ahead of the exponentials and the
+          // sums and packing PIPE columns behind, so that a single warp keeps
+          // the special-function unit busy
+          constexpr int PIPE = 16;
+#pragma unroll
+          for (int c = -PIPE; c < BKV + PIPE; c += 2) {
+            if (c + PIPE < BKV) scale_pair(r[c + PIPE], r[c + PIPE + 1], sc2, nm2);
+            if (c >= 0 && c < BKV) {
+              exp_in_place(r[c]);
+              exp_in_place(r[c + 1]);
+            }
+            if (c >= PIPE) {
+              const int d = c - PIPE;
+              sum_pair(sum2[(d >> 1) & 3], r[d], r[d + 1]);
+              r[d >> 1] = pack_pair(r[d], r[d + 1]);
+            }
+          }
+          float s0, s1, s2, s3, s4, s5, s6, s7;
+          unpack_f32x2(sum2[0], s0, s1);
+          unpack_f32x2(sum2[1], s2, s3);
+          unpack_f32x2(sum2[2], s4, s5);
+          unpack_f32x2(sum2[3], s6, s7);
+          bl = ((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7));
+          if (!__any_sync(0xffffffffu, bl > RAISE_SUM) || take_max) break;
+          take_max = true;
+        }
+        if (CAP) {
 #pragma unroll
           for (int q = 0; q < 8; ++q)
-            if (q < cap.n && cap.id[q] / BKV == kb0 + j)
-              cap_s[q] = __uint_as_float(tmem_ld1_nowait(tS0 + uint32_t(BKV) * uint32_t(g & 1) +
-                                                         lane_off + uint32_t(cap.id[q] % BKV))) *
-                         scale_log2;
-          tmem_wait_ld();
+            if (q < cap.n && cap.id[q] >= key0 && cap.id[q] < key0 + BKV) cap_s[q] *= scale_log2;
         }
-        tc_fence_before();
-        mbar_arrive(s_free + 8 * (g & 1));
-        // raw scores: the running max m is kept in scaled base-2 units; the
-        // scale (log2 e / sqrt(dh) > 0) commutes with the max, and
-        // p = 2^(s * scale - m) is one FFMA + ex2 per element
-        const int valid = Nk - (kb0 + j) * BKV;
-        if (valid < BKV) {  // the last, partial key block (warp-uniform)
-#pragma unroll
-          for (int c = 0; c < BKV; ++c)
-            if (c >= valid) r[c] = __float_as_uint(-INFINITY);
-        }
-        float mx8[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) mx8[q] = __uint_as_float(r[q]);
-#pragma unroll
-        for (int c = 8; c < BKV; ++c) mx8[c & 7] = fmaxf(mx8[c & 7], __uint_as_float(r[c]));
-        float mx = fmaxf(fmaxf(fmaxf(mx8[0], mx8[1]), fmaxf(mx8[2], mx8[3])),
-                         fmaxf(fmaxf(mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]))) * scale_log2;
-        // lazy rescale (warp-uniform decision: the TMEM accesses are
-        // warp-wide); O itself is rescaled below, once P V of the previous
-        // block has completed
-        bool rescale = false;
-        float alpha = 1.f;
-        if (j == 0) {
-          m = mx;
-        } else if (__any_sync(0xffffffffu, mx > m + LAZY_RESCALE)) {
-          rescale = true;
-          mx = fmaxf(mx, m);
-          alpha = ex2_ftz(m - mx);
+        if (take_max && i != (two ? 0 : x)) {
+          // O to the raised reference, once P V of the stream's previous block
+          // has completed
           l *= alpha;
-          m = mx;
-        }
-        // p = 2^(s scale - m): the scaling FMA and the row sum run two
-        // columns per instruction (packed f32x2)
-        const uint64_t sc2 = f32x2(scale_log2, scale_log2), nm2 = f32x2(-m, -m);
-        uint64_t sum2[4];
+          if (!mbar_sleep_warp(pv_done + 8 * (2 * x + ((cnt - 1) & 1)), ((cnt - 1) >> 1) & 1,
+                               abort_flag))
+            goto timeout;
+          tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) sum2[q] = f32x2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < BKV; c += 2) {
-          float a, b;
-          unpack_f32x2(fma_f32x2(f32x2(__uint_as_float(r[c]), __uint_as_float(r[c + 1])), sc2, nm2),
-                       a, b);
-          a = ex2_ftz(a);
-          b = ex2_ftz(b);
-          r[c] = __float_as_uint(a);
-          r[c + 1] = __float_as_uint(b);
-          sum2[(c >> 1) & 3] = add_f32x2(sum2[(c >> 1) & 3], f32x2(a, b));
-        }
-        float s0, s1, s2, s3, s4, s5, s6, s7;
-        unpack_f32x2(sum2[0], s0, s1);
-        unpack_f32x2(sum2[1], s2, s3);
-        unpack_f32x2(sum2[2], s4, s5);
-        unpack_f32x2(sum2[3], s6, s7);
-        l += ((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7));
-        // the P buffer and O are free once P V of the previous block is done
-        if (g > 0 && !mbar_sleep_warp(pv_done, (g - 1) & 1, abort_flag)) goto timeout;
-        tc_fence_after();
-        if (rescale) {
-#pragma unroll
-          for (int i = 0; i < C::DHP / 16; ++i) {
+          for (int c = 0; c < C::DHP / 16; ++c) {
             uint32_t o16[16];
-            tmem_ld16_nowait(tO + lane_off + 16u * i, o16);
+            tmem_ld16_nowait(to + 16u * c, o16);
             tmem_wait_ld();
 #pragma unroll
             for (int e = 0; e < 16; ++e) o16[e] = __float_as_uint(__uint_as_float(o16[e]) * alpha);
-            tmem_st16(tO + lane_off + 16u * i, o16);
+            tmem_st16(to + 16u * c, o16);
           }
         }
-        // P row (64 keys as 32 bf16 pairs): the A operand of P V
-        const uint32_t tp = tP + lane_off;
+        l += bl;
+        // P row (80 keys as 40 bf16 pairs) over S: the A operand of P V
 #pragma unroll
-        for (int h2 = 0; h2 < 2; ++h2) {
-          uint32_t w[16];
-#pragma unroll
-          for (int c = 0; c < 16; ++c)
-            w[c] = pack_bf16x2(__uint_as_float(r[32 * h2 + 2 * c]),
-                               __uint_as_float(r[32 * h2 + 2 * c + 1]));
-          tmem_st16(tp + 16u * h2, w);
-        }
+        for (int c = 0; c < BKV / 32; ++c) tmem_st16(ts + 16u * c, r + 16 * c);
+        if (BKV % 32) tmem_st8(ts + uint32_t(BKV / 32 * 16), r + BKV / 32 * 16);
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(p_ready);
+        arrive(p_ready + 8 * (2 * x + b));
       }
-      // ---- unit epilogue
+      // ---- end of the unit.  Two tiles: a thread has its row's whole O.
+      // One tile: the two streams' rows are merged, stream 0's thread taking
+      // a row's first columns, stream 1's the rest
+      float M = m, L = l, w0 = 1.f, w1 = 0.f;
+      if (!two) {
+        s_ml[uc & 1][x][row] = make_float2(m, l);
+        if (!join()) goto timeout;
+        const float2 ml = s_ml[uc & 1][x ^ 1][row];
+        // (a stream without a block has m = -inf, l = 0 and no O)
+        M = finite_max(fmaxf(m, ml.x));
+        const float wm = ex2_ftz(m - M), wo = ex2_ftz(ml.x - M);
+        L = l * wm + ml.y * wo;
+        w0 = x ? wo : wm;
+        w1 = x ? wm : wo;
+      }
       if (!mbar_sleep_warp(o_full, uc & 1, abort_flag)) goto timeout;
       tc_fence_after();
-      uint32_t o[C::DHP];
+      const int trow = (two ? x * BQ : 0) + row;  // row within the group
+      const bool live = trow < tl.rows;
+      bf16* orow = O + size_t(tl.row0 + trow) * ldo + w.h * DH;
+      const float inv = L > 0.f ? 1.f / L : 0.f;
+      constexpr int H0 = C::TAIL ? 40 : 32;  // columns of the first half; the second has 32
+      const uint32_t tb = tmem + TM_O + lane_off + (two ? TM_O_STEP * uint32_t(x) : 0u);
+      const bool shared = w.share >= 0;
+      const size_t slot = (size_t(max(w.share, 0)) * 2 + (two ? x : 0)) * (BQ * PART_STRIDE);
+      const int hf0 = two ? 0 : x, hf1 = two ? 2 : x + 1;
+      for (int hf = hf0; hf < hf1; ++hf) {
+        const int col0 = hf ? H0 : 0, ncol = hf ? DH - H0 : H0;
 #pragma unroll
-      for (int i = 0; i < C::DHP / 16; ++i) tmem_ld16_nowait(tO + lane_off + 16u * i, o + 16 * i);
-      tmem_wait_ld();
-      tc_fence_before();
-      mbar_arrive(o_free);
-      if (slot < 0) {
-        const TileLoc tl = locate_tile(rm, ai.n, D, qt);
-        const int qrow = tl.row0 + row;
-        if (cap.n && row < tl.rows) {
-          const int tok = rm.tok ? __ldg(rm.tok + qrow) : qrow;
-          const float inv_l = l > 0.f ? 1.f / l : 0.f;
+        for (int c = 0; c < H0; c += 8) {
+          if (c >= ncol) break;
+          uint32_t a[8], b[8];
+          float o[8];
+          tmem_ld8_nowait(tb + uint32_t(col0 + c), a);
+          if (!two && n > 1) tmem_ld8_nowait(tb + TM_O_STEP + uint32_t(col0 + c), b);
+          tmem_wait_ld();
 #pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (q < cap.n)
-              atomicAdd(cap.out + size_t(tok) * cap.ldo + cap.id[q],
-                        cap.w * ex2_ftz(cap_s[q] - m) * inv_l);
-        }
-        if (row < tl.rows) {
-          const float inv = l > 0.f ? 1.f / l : 0.f;
-          uint4* dst = reinterpret_cast<uint4*>(O + size_t(qrow) * ldo + h * DH);
-#pragma unroll
-          for (int c8 = 0; c8 < DH / 8; ++c8) {
-            uint4 w;
-            w.x = pack_bf16x2(__uint_as_float(o[8 * c8 + 0]) * inv, __uint_as_float(o[8 * c8 + 1]) * inv);
-            w.y = pack_bf16x2(__uint_as_float(o[8 * c8 + 2]) * inv, __uint_as_float(o[8 * c8 + 3]) * inv);
-            w.z = pack_bf16x2(__uint_as_float(o[8 * c8 + 4]) * inv, __uint_as_float(o[8 * c8 + 5]) * inv);
-            w.w = pack_bf16x2(__uint_as_float(o[8 * c8 + 6]) * inv, __uint_as_float(o[8 * c8 + 7]) * inv);
-            dst[c8] = w;
+          for (int e = 0; e < 8; ++e) {
+            o[e] = __uint_as_float(a[e]) * w0;
+            if (!two && n > 1) o[e] = fmaf(__uint_as_float(b[e]), w1, o[e]);
+          }
+          if (shared) {  // a share of the pair's keys: its planes to the workspace
+            float4* mine = reinterpret_cast<float4*>(part + slot) + ((col0 + c) / 4) * BQ + row;
+            __stcg(mine, make_float4(o[0], o[1], o[2], o[3]));
+            __stcg(mine + BQ, make_float4(o[4], o[5], o[6], o[7]));
+          } else if (live) {
+            *reinterpret_cast<uint4*>(orow + col0 + c) =
+                make_uint4(pack_bf16x2(o[0] * inv, o[1] * inv), pack_bf16x2(o[2] * inv, o[3] * inv),
+                           pack_bf16x2(o[4] * inv, o[5] * inv), pack_bf16x2(o[6] * inv, o[7] * inv));
           }
         }
-      } else {
-        // a piece of the pair's keys: unnormalised O with its row max and
-        // sum; the combine kernel merges the pieces
-        // (the workspace slot's planes: column group c4 of every row, then
-        // the rows' (max, sum); a warp's stores are whole 512-byte runs)
-        float* mine = part + (size_t(blockIdx.x) * 2 + slot) * (BQ * PART_STRIDE);
+      }
+      tc_fence_before();
+      arrive(o_free);
+      if (CAP && live) {  // the localisation scores of the listed keys (one share)
+        const int tok = rm.tok ? __ldg(rm.tok + tl.row0 + trow) : tl.row0 + trow;
 #pragma unroll
-        for (int c4 = 0; c4 < DH / 4; ++c4)
-          __stcg(reinterpret_cast<float4*>(mine) + c4 * BQ + row,
-                 make_float4(__uint_as_float(o[4 * c4]), __uint_as_float(o[4 * c4 + 1]),
-                             __uint_as_float(o[4 * c4 + 2]), __uint_as_float(o[4 * c4 + 3])));
-        __stcg(reinterpret_cast<float2*>(mine + DH * BQ) + row, make_float2(m, l));
+        for (int q = 0; q < 8; ++q)
+          if (q < cap.n && (two || ((cap.id[q] / BKV) & 1) == x))  // this stream's block held it
+            atomicAdd(cap.out + size_t(tok) * cap.ldo + cap.id[q],
+                      cap.w * ex2_ftz(cap_s[q] - M) * inv);
+      }
+      if (shared) {
+        // the last of the pair's units merges them all
+        if (two || x == 0)
+          __stcg(reinterpret_cast<float2*>(part + slot + DH * BQ) + row, make_float2(M, L));
+        __threadfence();
+        if (!join()) goto timeout;
+        if (threadIdx.x == 128) {
+          unsigned* tk = ticket + (w.pair - un.whole);
+          const unsigned t = atomicAdd(tk, 1u);
+          s_last = t == unsigned(un.split) - 1u;
+          if (s_last) *tk = 0u;  // for the next launch
+          __threadfence();
+        }
+        if (!join()) goto timeout;
+        if (!s_last) continue;
+        const float* base = part + (size_t(w.pair - un.whole) * un.split * 2 + (two ? x : 0)) *
+                                       (BQ * PART_STRIDE);
+        auto piece = [&](int q) { return base + size_t(q) * (2 * BQ * PART_STRIDE); };
+        float Mt = -INFINITY;
+#pragma unroll 4
+        for (int q = 0; q < un.split; ++q)
+          Mt = fmaxf(Mt, __ldcg(reinterpret_cast<const float2*>(piece(q) + DH * BQ) + row).x);
+        Mt = finite_max(Mt);
+        for (int hf = hf0; hf < hf1; ++hf) {
+          // a half row's columns of two shares in flight at a time
+          const int col0 = hf ? H0 : 0, ncol = hf ? DH - H0 : H0;
+          float o[H0], Lt = 0.f;
+#pragma unroll
+          for (int c = 0; c < H0; ++c) o[c] = 0.f;
+#pragma unroll 2
+          for (int q = 0; q < un.split; ++q) {
+            const float2 mq = __ldcg(reinterpret_cast<const float2*>(piece(q) + DH * BQ) + row);
+            const float4* b = reinterpret_cast<const float4*>(piece(q)) + (col0 / 4) * BQ + row;
+            float4 v[H0 / 4];
+#pragma unroll
+            for (int c4 = 0; c4 < H0 / 4; ++c4)
+              if (4 * c4 < ncol) v[c4] = __ldcg(b + c4 * BQ);
+            const float wq = ex2_ftz(mq.x - Mt);
+            Lt += wq * mq.y;
+#pragma unroll
+            for (int c4 = 0; c4 < H0 / 4; ++c4)
+              if (4 * c4 < ncol) {
+                o[4 * c4] = fmaf(wq, v[c4].x, o[4 * c4]);
+                o[4 * c4 + 1] = fmaf(wq, v[c4].y, o[4 * c4 + 1]);
+                o[4 * c4 + 2] = fmaf(wq, v[c4].z, o[4 * c4 + 2]);
+                o[4 * c4 + 3] = fmaf(wq, v[c4].w, o[4 * c4 + 3]);
+              }
+          }
+          const float inv_t = Lt > 0.f ? 1.f / Lt : 0.f;
+#pragma unroll
+          for (int c = 0; c < H0; c += 8)
+            if (c < ncol && live)
+              *reinterpret_cast<uint4*>(orow + col0 + c) = make_uint4(
+                  pack_bf16x2(o[c] * inv_t, o[c + 1] * inv_t),
+                  pack_bf16x2(o[c + 2] * inv_t, o[c + 3] * inv_t),
+                  pack_bf16x2(o[c + 4] * inv_t, o[c + 5] * inv_t),
+                  pack_bf16x2(o[c + 6] * inv_t, o[c + 7] * inv_t));
+        }
       }
     }
   }
@@ -614,7 +796,7 @@ done:
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, TMEM_COLS);
+    tmem_dealloc(tmem, TMEM_COLS);
   }
 }
 
@@ -1094,89 +1276,6 @@ xf_done:
   }
 }
 
-// Merge of the pieces of the pairs that stream-K cut.  The pieces of a pair
-// come from CTAs cta_of(first block) .. cta_of(last block); a CTA's piece is
-// its first (slot 0) when its range starts inside the pair, else its last
-// (slot 1).  A workspace slot holds its piece as DH / 4 planes of 128 float4
-// (head-dim columns 4 c .. 4 c + 3 of the tile's rows), then the rows' (max,
-// sum) pairs, so that the attention kernel's softmax threads (one row each)
-// and this kernel's lanes (one row each) access whole 512-byte runs.  A work
-// unit is 32 consecutive rows of one cut pair and COMBINE_CH of the column
-// planes; units go to warps in turn.  Per row: the largest of the pieces'
-// maxima M, then the pieces' columns weighted by 2^(m_q - M), over the
-// weighted sums, stored as bf16.  Each of the two passes keeps several
-// pieces' loads in flight.
-constexpr int COMBINE_THREADS = 256, COMBINE_CH = 3;
-template <int DH>
-__global__ void __launch_bounds__(COMBINE_THREADS, 2)
-attn_combine_kernel(const float* __restrict__ part, bf16* __restrict__ O, int ldo, int heads,
-                    RowMap rm, int n_items, int Nk, int attn_grid, unsigned* err) {
-  // the row count predates the attention launch (see attn_tc_kernel): read
-  // before the wait; the pieces come from the predecessor
-  const int D = live_count(rm.count, rm.bound, err);
-  AttnSched sc;
-  sc.init(query_tiles(rm, n_items, D), heads, Nk, attn_grid);
-  pdl_wait();
-  pdl_trigger();
-  if (!sc.streamk) return;
-  constexpr int C4 = DH / 4, NCH = (C4 + COMBINE_CH - 1) / COMBINE_CH;
-  constexpr int PER_PAIR = (BQ / 32) * NCH;  // units of one pair
-  const int lane = threadIdx.x & 31;
-  const int units = sc.pairs * PER_PAIR;
-  const int nwarps = int(gridDim.x) * (COMBINE_THREADS / 32);
-  for (int u = int(blockIdx.x) * (COMBINE_THREADS / 32) + (int(threadIdx.x) >> 5); u < units;
-       u += nwarps) {
-    const int pair = u / PER_PAIR, rest = u - pair * PER_PAIR;
-    const int row = (rest / NCH) * 32 + lane, c0 = (rest - (rest / NCH) * NCH) * COMBINE_CH;
-    const int lo = pair * sc.nkb;
-    const int c_lo = sc.cta_of(lo);
-    const int np = sc.cta_of(lo + sc.nkb - 1) - c_lo + 1;
-    if (np == 1) continue;  // one CTA held the whole pair (warp-uniform)
-    const int slot_lo = sc.bound(c_lo) == lo ? 0 : 1;
-    const TileLoc tl = locate_tile(rm, n_items, D, pair % sc.qtiles);
-    const int h = pair / sc.qtiles;
-    auto slot = [&](int q) {
-      return part + (size_t(c_lo + q) * 2 + (q == 0 ? slot_lo : 0)) * (BQ * PART_STRIDE);
-    };
-    float M = -INFINITY;
-#pragma unroll 8
-    for (int q = 0; q < np; ++q)
-      M = fmaxf(M, __ldcg(reinterpret_cast<const float2*>(slot(q) + DH * BQ) + row).x);
-    float L = 0.f;
-    float4 acc[COMBINE_CH];
-#pragma unroll
-    for (int c = 0; c < COMBINE_CH; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 4
-    for (int q = 0; q < np; ++q) {
-      const float* b = slot(q);
-      const float2 ml = __ldcg(reinterpret_cast<const float2*>(b + DH * BQ) + row);
-      float4 v[COMBINE_CH];
-#pragma unroll
-      for (int c = 0; c < COMBINE_CH; ++c)
-        if (c0 + c < C4) v[c] = __ldcg(reinterpret_cast<const float4*>(b) + (c0 + c) * BQ + row);
-      const float wq = ex2_ftz(ml.x - M);
-      L += wq * ml.y;
-#pragma unroll
-      for (int c = 0; c < COMBINE_CH; ++c)
-        if (c0 + c < C4) {
-          acc[c].x += wq * v[c].x;
-          acc[c].y += wq * v[c].y;
-          acc[c].z += wq * v[c].z;
-          acc[c].w += wq * v[c].w;
-        }
-    }
-    if (row < tl.rows) {
-      const float inv = L > 0.f ? 1.f / L : 0.f;
-      uint2* dst = reinterpret_cast<uint2*>(O + size_t(tl.row0 + row) * ldo + h * DH) + c0;
-#pragma unroll
-      for (int c = 0; c < COMBINE_CH; ++c)
-        if (c0 + c < C4)
-          dst[c] = make_uint2(pack_bf16x2(acc[c].x * inv, acc[c].y * inv),
-                              pack_bf16x2(acc[c].z * inv, acc[c].w * inv));
-    }
-  }
-}
-
 // ------------------------------------------------------------------- host
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -1247,38 +1346,50 @@ int device_sms_attn() {
   if (!sms[dev]) {
     int v = 0;
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaFuncSetAttribute(attn_tc_kernel<72>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(ACfg<72>::SMEM)) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(ACfg<64>::SMEM)) != cudaSuccess ||
-        cudaFuncSetAttribute(xattn_tc_kernel<72, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XCfg<72>::SMEM)) !=
+    const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    if (cudaFuncSetAttribute(attn_tc_kernel<72, false>, smem, int(ACfg<72>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(attn_tc_kernel<72, true>, smem, int(ACfg<72>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(attn_tc_kernel<64, false>, smem, int(ACfg<64>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(attn_tc_kernel<64, true>, smem, int(ACfg<64>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(xattn_tc_kernel<72, false>, smem, int(XCfg<72>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(xattn_tc_kernel<72, true>, smem, int(XCfg<72>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(xattn_tc_kernel<64, false>, smem, int(XCfg<64>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(xattn_tc_kernel<64, true>, smem, int(XCfg<64>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(xfused_tc_kernel<72, false>, smem, int(XFCfg<72>::SMEM)) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(xattn_tc_kernel<72, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XCfg<72>::SMEM)) !=
+        cudaFuncSetAttribute(xfused_tc_kernel<72, true>, smem, int(XFCfg<72>::SMEM)) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(xattn_tc_kernel<64, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XCfg<64>::SMEM)) !=
+        cudaFuncSetAttribute(xfused_tc_kernel<64, false>, smem, int(XFCfg<64>::SMEM)) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(xattn_tc_kernel<64, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XCfg<64>::SMEM)) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(xfused_tc_kernel<72, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XFCfg<72>::SMEM)) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(xfused_tc_kernel<72, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XFCfg<72>::SMEM)) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(xfused_tc_kernel<64, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XFCfg<64>::SMEM)) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(xfused_tc_kernel<64, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(XFCfg<64>::SMEM)) !=
+        cudaFuncSetAttribute(xfused_tc_kernel<64, true>, smem, int(XFCfg<64>::SMEM)) !=
             cudaSuccess)
       return 0;
     sms[dev] = v;
   }
   return sms[dev];
+}
+
+// The plans of a (heads, keys) shape, cached.  With a capture every key sits in
+// one unit.
+PlanTable plan_table(int heads, int Nk, int grid, bool capture) {
+  static std::mutex mu;
+  static std::unordered_map<uint64_t, PlanTable> cache;
+  if (capture) return PlanTable{};
+  const uint64_t key = (uint64_t(heads) << 40) | (uint64_t(grid) << 32) | uint64_t(unsigned(Nk));
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = cache.find(key);
+  if (it != cache.end()) return it->second;
+  PlanTable t{};
+  for (int tiles = 1; tiles <= 2; ++tiles)
+    for (int i = 0; i < PLAN_TABLE; ++i) {
+      int cost;
+      t.split[tiles - 1][i] =
+          uint8_t(pick_split((i + 1) * heads, (Nk + BKV - 1) / BKV, grid, tiles, &cost));
+      t.cost[tiles - 1][i] = uint16_t(cost < 65535 ? cost : 65535);
+    }
+  if (cache.size() > 1024) cache.clear();
+  cache.emplace(key, t);
+  return t;
 }
 
 }  // namespace
@@ -1288,7 +1399,11 @@ size_t attention_split_floats(int Nmax, int heads, int dh) {
   (void)heads;
   (void)dh;
   const int sms = device_sms_attn();
-  return size_t(8) * (sms > 0 ? sms : 160) * BQ * PART_STRIDE;
+  return size_t(SLOTS_PER_SM) * (sms > 0 ? sms : 160) * BQ * PART_STRIDE;
+}
+size_t attention_tickets() {
+  const int sms = device_sms_attn();
+  return size_t(SLOTS_PER_SM) * (sms > 0 ? sms : 160);
 }
 
 
@@ -1304,19 +1419,16 @@ cudaError_t launch_attention(const bf16* Q, int ldq, const bf16* K, const bf16* 
       return cudaErrorInvalidValue;
   const int sms = device_sms_attn();
   if (!sms) return cudaErrorInvalidDevice;
-  // a 64-wide 128B-swizzled map and a 16-wide 32B-swizzled tail map per operand
-  CUtensorMap tq, tqt, tk, tkt, tv;
+  // 64-wide 128B-swizzled maps, and a 16-wide 32B-swizzled one for Q's tail
+  CUtensorMap tq, tqt, tk, tv;
   RC_TRY(head_map(Q, rm.bound, ldq, heads, dh, 64, BQ, &tq));
   RC_TRY(head_map(K, kv_rows, ldkv, heads, dh, 64, BKV, &tk));
   RC_TRY(head_map(V, kv_rows, ldkv, heads, dh, 64, BKV, &tv));
   RC_TRY(head_map(Q, rm.bound, ldq, heads, dh, 16, BQ, &tqt));
-  RC_TRY(head_map(K, kv_rows, ldkv, heads, dh, 16, BKV, &tkt));
   const float scale_log2 = float(1.4426950408889634 / sqrt(double(dh)));
   AttnCapture cap{};
   if (capture && capture->n > 0) {
-    // every key must sit in the one unit of its (query tile, head)
-    if (capture->n > 8 || !capture->out || (Nk + BKV - 1) / BKV >= 2 * MIN_KB_PER_SPLIT)
-      return cudaErrorInvalidValue;
+    if (capture->n > 8 || !capture->out || Nk > CAPTURE_KEYS) return cudaErrorInvalidValue;
     for (int q = 0; q < capture->n; ++q)
       if (capture->id[q] < 0 || capture->id[q] >= Nk || capture->id[q] >= capture->ldo)
         return cudaErrorInvalidValue;
@@ -1339,34 +1451,19 @@ cudaError_t launch_attention(const bf16* Q, int ldq, const bf16* K, const bf16* 
     count_launches(1);
     return cudaSuccess;
   }
-  const int grid = CTAS_PER_SM * sms;
+  const PlanTable plan = plan_table(heads, Nk, sms, cap.n > 0);
+  if (as.part_floats < size_t(SLOTS_PER_SM) * sms * BQ * PART_STRIDE || !as.ticket)
+    return cudaErrorInvalidValue;
   {
     const unsigned long long tiles = (rm.bound + BQ - 1) / BQ + ai.n - 1;
-    if (tiles * heads * ((Nk + BKV - 1) / BKV) * grid >= (1ull << 32)) return cudaErrorInvalidValue;
+    if (tiles * heads * MAX_SPLIT >= (1ull << 31)) return cudaErrorInvalidValue;
   }
-  // two partial pieces per CTA at most
-  if (as.part_floats < size_t(2) * grid * BQ * PART_STRIDE) return cudaErrorInvalidValue;
-  if (dh == 72)
-    RC_TRY(launch_k(attn_tc_kernel<72>, dim3(grid), dim3(THREADS), ACfg<72>::SMEM, st, tq, tqt,
-                    tk, tkt, tv, ai, Nk, O, ldo, heads, rm, scale_log2, err, as.part, cap));
-  else
-    RC_TRY(launch_k(attn_tc_kernel<64>, dim3(grid), dim3(THREADS), ACfg<64>::SMEM, st, tq, tqt,
-                    tk, tkt, tv, ai, Nk, O, ldo, heads, rm, scale_log2, err, as.part, cap));
+  auto fn = dh == 72 ? (cap.n ? attn_tc_kernel<72, true> : attn_tc_kernel<72, false>)
+                     : (cap.n ? attn_tc_kernel<64, true> : attn_tc_kernel<64, false>);
+  RC_TRY(launch_k(fn, dim3(sms), dim3(THREADS), dh == 72 ? ACfg<72>::SMEM : ACfg<64>::SMEM, st, tq,
+                  tqt, tk, tv, K, V, ldkv, kv_rows, ai, plan, Nk, O, ldo, heads, rm, scale_log2,
+                  err, as.part, as.ticket, cap));
   count_launches(1);
-  // stream-K (and so partial pieces) only with at least 2 MIN_KB_PER_SPLIT key blocks
-  if ((Nk + BKV - 1) / BKV >= 2 * MIN_KB_PER_SPLIT) {
-    const int tiles = (rm.bound + BQ - 1) / BQ + ai.n - 1;  // bound of the query tiles
-    // units of 32 rows and COMBINE_CH column planes of a pair
-    const int units = tiles * heads * (BQ / 32) * ((dh / 4 + COMBINE_CH - 1) / COMBINE_CH);
-    const int cgrid = min((units + COMBINE_THREADS / 32 - 1) / (COMBINE_THREADS / 32), 2 * sms);
-    if (dh == 72)
-      RC_TRY(launch_k(attn_combine_kernel<72>, dim3(cgrid), dim3(COMBINE_THREADS), 0, st,
-                      as.part, O, ldo, heads, rm, ai.n, Nk, grid, err));
-    else
-      RC_TRY(launch_k(attn_combine_kernel<64>, dim3(cgrid), dim3(COMBINE_THREADS), 0, st,
-                      as.part, O, ldo, heads, rm, ai.n, Nk, grid, err));
-    count_launches(1);
-  }
   return cudaSuccess;
 }
 

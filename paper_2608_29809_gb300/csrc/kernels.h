@@ -158,8 +158,10 @@ cudaError_t launch_gemm(const bf16* A, int lda, const bf16* W, int Mbound, const
 struct AttnScratch {
   float* part;
   size_t part_floats;
+  unsigned* ticket;  // attention_tickets() of them, zero between launches
 };
 size_t attention_split_floats(int Nmax, int heads, int dh);
+size_t attention_tickets();
 
 // Per-item key / value placement of one attention launch: item i's keys are
 // rows krow[i] .. krow[i] + Nk - 1 of K (values likewise from vrow[i] of V).

@@ -231,7 +231,7 @@ void free_ctx(rc_ctx* c) {
   probe_free(c);
   void* ps[] = {c->xf,   c->xb,   c->ob,   c->q,    c->u,      c->fbuf,
                 c->h1,   c->temb, c->tb,   c->iota, c->b_tok,  c->b_item,
-                c->b_meta, c->err, c->wait_flag, c->as.part, c->temb_tab, c->tb_tab};
+                c->b_meta, c->err, c->wait_flag, c->as.part, c->as.ticket, c->temb_tab, c->tb_tab};
   for (void* p : ps)
     if (p) cudaFree(p);
   delete c;
@@ -521,7 +521,8 @@ rc_status rc_create(const rc_dims* dims, rc_ctx** out) {
     return s;
   }
   c->as.part_floats = rc::attention_split_floats(int(N), D.heads, dh);
-  if ((s = dalloc(&c->as.part, c->as.part_floats, "attn part"))) {
+  if ((s = dalloc(&c->as.part, c->as.part_floats, "attn part")) ||
+      (s = dalloc(&c->as.ticket, rc::attention_tickets(), "attn tickets"))) {
     free_ctx(c);
     return s;
   }
@@ -529,6 +530,8 @@ rc_status rc_create(const rc_dims* dims, rc_ctx** out) {
   rc::count_launches(1);
   cudaError_t e = cudaMemset(c->err, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemset(c->wait_flag, 0, sizeof(unsigned));
+  if (e == cudaSuccess)
+    e = cudaMemset(c->as.ticket, 0, rc::attention_tickets() * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     free_ctx(c);
@@ -1533,6 +1536,9 @@ rc_status rc_sync(rc_ctx* c, rc_stream stream) {
   RC_CUDA(cudaMemcpy(&w, c->err, sizeof(w), cudaMemcpyDeviceToHost), "read error word");
   if (w) {
     RC_CUDA(cudaMemset(c->err, 0, sizeof(unsigned)), "clear error word");
+    // (a launch that gave up may have left some of its tickets)
+    RC_CUDA(cudaMemset(c->as.ticket, 0, rc::attention_tickets() * sizeof(unsigned)),
+            "clear tickets");
     if (w & rc::DEVERR_TIMEOUT) return fail(RC_ERR_TIMEOUT, "a bounded device wait gave up");
     return fail(RC_ERR_DEVICE_ASSERT, "device check failed (bits 0x%x: %s%s)", w,
                 (w & rc::DEVERR_INDEX) ? "index out of range " : "",
