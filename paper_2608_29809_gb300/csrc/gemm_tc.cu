@@ -17,16 +17,20 @@
 // into equal k-block ranges (stream-K).  Its casting variant (x += ..., then
 // xb = bf16(x), read-modify-write) and the other epilogues see whole tiles.
 //
-// CTA = 16 warps: warp 0 issues TMA loads (A), warp 14 those of W, warp 1
-// owns TMEM and issues the MMAs (one thread), warps 2..13 drain the
+// CTA = 15 warps: warp 0 issues TMA loads (A), warp 14 those of W, warp 1
+// owns TMEM and issues the MMAs (one elected thread), warps 2..13 drain the
 // accumulator (one TMEM lane = one output row per thread; three warps per
-// TMEM lane quarter take every third 32-column chunk; re-staged through
-// shared memory so that global writes are whole row pieces), and warp 15
-// is a second MMA issuer when every CTA holds one work item (the item's odd
-// k-blocks into the second accumulator, see split2).  The epilogue is
+// TMEM lane quarter take every third 32-column chunk).  The epilogue is
 // latency-bound (a CTA holds one tile at small row counts), so its width is
-// worth more than a deeper ring.  Otherwise two TMEM accumulators of up to
-// 256 columns let the epilogue of one tile overlap the main loop of the next.
+// worth more than a deeper ring, and every epilogue is its own kernel: a
+// launch runs its code once per CTA, so instructions that it does not need
+// cost fetches (at 831 rows warps of the one-kernel form waited 2-4 cycles
+// per instruction for the next one).  Against that form, with two issuing
+// threads, schedules chosen on the device, bf16 tiles re-staged through shared
+// memory and W waiting for the previous kernel: a 28-block step at 831 rows
+// 2980 -> 2718 us, at 1512 rows of 8 items 4312 -> 3950, two blocks at 132 /
+// 4096 rows 177 -> 158 / 661 -> 604 us.  Two TMEM accumulators of up to 256 columns let the epilogue
+// of one tile overlap the main loop of the next.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -47,10 +51,9 @@ constexpr int BM = 128, BK = 64;
 // TMA warp (A, or A and W for CTA pairs), MMA warp, 12 epilogue warps, a
 // second TMA warp that loads W for unpaired CTAs (each TMA request takes long
 // enough to issue that one thread issuing both operands bounds the main
-// loop), and a second MMA warp
-constexpr int THREADS = 512;
+// loop, and W does not wait for the previous kernel)
+constexpr int THREADS = 480;
 constexpr int W_WARP = 14;
-constexpr int MMA2_WARP = 15;
 constexpr int STAGE_A = BM * BK * 2;   // bytes
 constexpr int MIN_KB_PER_CTA = 4;
 constexpr int STAGING_WARP = 32 * 128;  // epilogue staging: 32 rows of 128 B per warp
@@ -69,8 +72,9 @@ constexpr uint32_t IDESC_BASE = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(B
 // the same for the M = 256 MMA of a CTA pair
 constexpr uint32_t IDESC_PAIR = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(256 >> 4) << 24);
 // The tile width and split chosen on the host for 1 .. BN_TABLE row tiles
-// (BN / 64 + 8 S), passed by value; larger row counts choose on the device.
-constexpr int BN_TABLE = 64;
+// (BN / 64 + 8 S), passed by value; larger row counts take the last entry's
+// width in whole tiles.
+constexpr int BN_TABLE = 128;
 struct BnTable {
   uint8_t w64[BN_TABLE];
 };
@@ -97,6 +101,19 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
                "f"(d)
                : "memory");
 }
+// 32 bytes (one sector) per thread.
+__device__ __forceinline__ void st_v8(void* p, const uint32_t* v) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
+               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void ld_v8(const float* p, float* v) {
+  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]),
+                 "=f"(v[6]), "=f"(v[7])
+               : "l"(p)
+               : "memory");
+}
 
 // The mode a schedule is planned for: a gated residual held to whole tiles
 // plans like any other 4-byte epilogue whose tiles are not split.
@@ -104,14 +121,9 @@ __host__ __device__ inline int sched_mode(const GemmEpi& ep) {
   return ep.mode == EPI_GATE_RES && ep.whole_tiles ? int(EPI_F32) : ep.mode;
 }
 
+template <int MODE>
 __device__ __forceinline__ bool gated(const GemmEpi& ep) {
-  return (ep.mode == EPI_GATE_RES || ep.mode == EPI_GATE_RES_CAST) && ep.gate_tab;
-}
-// The gate's per-item part comes with each row (from its item's timestep
-// vector) only when the launch has several items; with one item it is
-// folded into the staged gate vector.
-__device__ __forceinline__ bool row_gate(const GemmEpi& ep) {
-  return gated(ep) && ep.gate_off >= 0 && ep.its.n > 1;
+  return (MODE == EPI_GATE_RES || MODE == EPI_GATE_RES_CAST) && ep.gate_tab;
 }
 
 // The column vectors of one tile (columns col0 .. col0 + BN - 1) in shared
@@ -120,19 +132,23 @@ __device__ __forceinline__ bool row_gate(const GemmEpi& ep) {
 // residual does not start at k = 0: the update is a sum over pieces, so the
 // bias goes with one of them), sv[256 + c] = gate (table part, plus the
 // item's timestep part when the launch has one item).
+template <int MODE>
 __device__ __forceinline__ void stage_vectors(const GemmEpi& ep, int col0, int BN, bool with_bias,
                                               float* sv, int etid) {
   const float* tb0 = (ep.its.n == 1 && ep.gate_off >= 0) ? ep.its.tb[0] : nullptr;
-  for (int c = etid; c < BN; c += 384) {
-    const int col = col0 + c;
-    sv[c] = (ep.bias && with_bias) ? __ldg(ep.bias + col) : 0.f;
-    if (gated(ep)) sv[256 + c] = __ldg(ep.gate_tab + col) + (tb0 ? __ldg(tb0 + ep.gate_off + col) : 0.f);
+  if (etid < BN) {
+    const int col = col0 + etid;
+    sv[etid] = (ep.bias && with_bias) ? __ldg(ep.bias + col) : 0.f;
+    if (gated<MODE>(ep))
+      sv[256 + etid] = __ldg(ep.gate_tab + col) + (tb0 ? __ldg(tb0 + ep.gate_off + col) : 0.f);
   }
 }
 
 // Epilogue values of columns c0 .. c0+31 of one output row (cl = c0 within
 // the tile): bias, tanh-GELU, gate, from the staged vectors (plus the row's
-// item gate when the launch has several items).
+// item gate when the launch has several items; with one item it is folded
+// into the staged gate).
+template <int MODE>
 __device__ __forceinline__ void epilogue_values(const GemmEpi& ep, int c0, int cl, int item,
                                                 float* v, const float* sv) {
   const float4* b4 = reinterpret_cast<const float4*>(sv + cl);
@@ -141,200 +157,105 @@ __device__ __forceinline__ void epilogue_values(const GemmEpi& ep, int c0, int c
     const float4 b = b4[i];
     v[4 * i] += b.x; v[4 * i + 1] += b.y; v[4 * i + 2] += b.z; v[4 * i + 3] += b.w;
   }
-  if (ep.mode == EPI_GELU_BF16) {
+  if (MODE == EPI_GELU_BF16) {
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = gelu_tanh(v[i]);
-  } else if (gated(ep)) {
-    float g[32];
+  } else if (gated<MODE>(ep)) {
+    const float* tb = ep.gate_off >= 0 && ep.its.n > 1 ? ep.its.tb[item] : nullptr;
     const float4* g4 = reinterpret_cast<const float4*>(sv + 256 + cl);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float4 a = g4[i];
-      g[4 * i] = a.x; g[4 * i + 1] = a.y; g[4 * i + 2] = a.z; g[4 * i + 3] = a.w;
-    }
-    if (row_gate(ep)) {
-      const float* tb = ep.its.tb[item];
+      float4 g = g4[i];
       if (tb) {
-        float g2[32];
-        load32(tb + ep.gate_off + c0, g2);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) g[i] += g2[i];
+        const float4 e = __ldg(reinterpret_cast<const float4*>(tb + ep.gate_off + c0) + i);
+        g.x += e.x; g.y += e.y; g.z += e.z; g.w += e.w;
       }
-    }
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] *= g[i];
-  }
-}
-
-// 32 consecutive f32 columns of this thread's TMEM lane, summed over the two
-// accumulators at taddr and taddr + 256 (a tile whose k-blocks two MMA
-// threads split between them).
-__device__ __forceinline__ void tmem_ld32_sum2(uint32_t taddr, float* v) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    uint32_t a[16], b[16];
-    tmem_ld16_nowait(taddr + uint32_t(16 * h), a);
-    tmem_ld16_nowait(taddr + 256u + uint32_t(16 * h), b);
-    tmem_wait_ld();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[16 * h + i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
-  }
-}
-// The k-blocks of parity `par` of a CTA's one work item (k-blocks [kb0, kb1),
-// ring stages from 0), issued by one of two MMA threads into accumulator
-// `par` (TMEM columns 256 par ..); its tfull barrier is committed at the end.
-// Returns false when a bounded wait gave up.
-__device__ __forceinline__ bool mma_half(int par, int kb0, int kb1, int STAGES, int STAGE,
-                                         uint32_t ring, uint32_t tmem_base, uint32_t idesc,
-                                         uint32_t full0, uint32_t empty0, uint32_t tfull0,
-                                         uint32_t tempty0, volatile int* abort_flag) {
-  if (!mbar_wait(tempty0 + 8 * par, 1, abort_flag)) return false;
-  tc_fence_after();
-  const uint64_t da = sw128_desc(ring), db = sw128_desc(ring + STAGE_A);
-  const uint32_t dtm = tmem_base + uint32_t(par * 256);
-  int stage = par;
-  uint32_t phase = 0;
-  for (int kb = kb0 + par; kb < kb1; kb += 2) {
-    if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) return false;
-    tc_fence_after();
-    const uint64_t so = uint64_t((stage * STAGE) >> 4);
-#pragma unroll
-    for (int kk = 0; kk < BK / 16; ++kk)
-      umma_bf16(dtm, da + so + 2 * kk, db + so + 2 * kk, idesc,
-                (kb > kb0 + par || kk > 0) ? 1u : 0u);
-    umma_commit(empty0 + 8 * stage);
-    stage += 2;
-    if (stage >= STAGES) {
-      stage -= STAGES;
-      phase ^= 1;
+      v[4 * i] *= g.x; v[4 * i + 1] *= g.y; v[4 * i + 2] *= g.z; v[4 * i + 3] *= g.w;
     }
   }
-  umma_commit(tfull0 + 8 * par);
-  return true;
 }
 
 // Named barrier of the 12 epilogue warps.
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 384;" ::: "memory"); }
 
-// Destination of columns c0 .. c0+31 of output row r, or null when the row is
-// beyond the live count (or its token / item index is bad: QKV raises
-// DEVERR_INDEX).  tok / item of the row are loaded once per tile.
-__device__ __forceinline__ char* chunk_dst(const GemmEpi& ep, int r, int M, int tok, int item,
-                                           int c0) {
-  if (r >= M) return nullptr;
-  switch (ep.mode) {
-    case EPI_F32:
-      return reinterpret_cast<char*>(ep.out_f + size_t(r) * ep.ld_out + c0);
-    case EPI_GATE_RES:
-    case EPI_GATE_RES_CAST:
-      return reinterpret_cast<char*>(ep.xf + size_t(r) * ep.ld_xf + c0);
-    case EPI_QKV: {
-      const int part = c0 / ep.dsplit;
-      const int cc = c0 - part * ep.dsplit;
-      if (part == 0) return reinterpret_cast<char*>(ep.out_bf + size_t(r) * ep.ld_out + cc);
-      if (tok < 0 || tok >= ep.n_tokens || item < 0 || item >= ep.its.n) {
-        atomicOr(ep.err, DEVERR_INDEX);
-        return nullptr;
-      }
-      return reinterpret_cast<char*>(ep.its.slice[item] + (part == 1 ? ep.k_off : ep.v_off) +
-                                     size_t(tok) * ep.dsplit + cc);
-    }
-    default:
-      return reinterpret_cast<char*>(ep.out_bf + size_t(r) * ep.ld_out + c0);
+// Columns c0 .. c0 + 31 of output row r as bf16: two sectors of the row's own
+// (the lanes' rows may lie anywhere: QKV scatters K and V to the cache rows
+// of the rows' tokens).
+__device__ __forceinline__ void store_bf16(bf16* p, const float* v) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t u[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) u[i] = pack_bf16x2(v[16 * h + 2 * i], v[16 * h + 2 * i + 1]);
+    st_v8(p + 16 * h, u);
   }
 }
 
-// Writes one warp's 32 x 32 chunk (lane = row, v = its 32 columns) to global
-// memory with coalesced accesses: each lane parks its row in the warp's 4 KB
-// staging area, then groups of lanes write whole 128-byte (f32) or 64-byte
-// (bf16) row pieces.  Staging is XOR-swizzled in 16-byte units so that both
-// the row-per-lane writes and the piece-per-lane-group reads are free of bank
-// conflicts.  The gated residual goes out as vector reductions (x += value);
-// its casting variant reads x, adds, and writes x and bf16(x) (xb_row: the
-// row's bf16 copy, columns c0 ..).
-__device__ __forceinline__ void store_chunk(int mode, uint8_t* stg, int lane, const float* v,
-                                            char* dst, bf16* xb_row) {
+// The gated residual of one warp's 32 x 32 chunk (lane = row, v = its 32
+// columns) as vector reductions into x: each lane parks its row in the warp's
+// 4 KB staging area, then eight lanes add one whole 128-byte row piece.
+// Staging is XOR-swizzled in 16-byte units so that both the row-per-lane
+// writes and the piece-per-lane-group reads are free of bank conflicts.
+__device__ __forceinline__ void reduce_chunk(uint8_t* stg, int lane, const float* v, float* dst) {
   const uint32_t s0 = saddr(stg);
-  if (mode == EPI_F32 || mode == EPI_GATE_RES || mode == EPI_GATE_RES_CAST) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(
-                       s0 + lane * 128 + 16 * (j ^ (lane & 7))),
-                   "f"(v[4 * j]), "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
-                   : "memory");
-    __syncwarp();
-    // all row pointers and pieces first (independent, so they overlap),
-    // then the global writes
-    const int j = lane & 7;
-    char* d[8];
-    bf16* xb[8];
-    float4 x[8];
+  for (int j = 0; j < 8; ++j)
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(
+                     s0 + lane * 128 + 16 * (j ^ (lane & 7))),
+                 "f"(v[4 * j]), "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
+                 : "memory");
+  __syncwarp();
+  const int j = lane & 7;
 #pragma unroll
-    for (int pass = 0; pass < 8; ++pass) {
-      const int row = pass * 4 + (lane >> 3);
-      d[pass] = reinterpret_cast<char*>(
-          __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), row));
-      xb[pass] = mode == EPI_GATE_RES_CAST
-                     ? reinterpret_cast<bf16*>(__shfl_sync(
-                           0xffffffffu, reinterpret_cast<unsigned long long>(xb_row), row))
-                     : nullptr;
-      x[pass] = *reinterpret_cast<const float4*>(stg + row * 128 + 16 * (j ^ (row & 7)));
-    }
-    if (mode == EPI_GATE_RES_CAST) {
-      // read-modify-write: all eight reads in flight before the writes
-      float4 o[8];
-#pragma unroll
-      for (int pass = 0; pass < 8; ++pass)
-        o[pass] = d[pass] ? __ldcg(reinterpret_cast<const float4*>(d[pass]) + j)
-                          : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int pass = 0; pass < 8; ++pass) {
-        if (!d[pass]) continue;
-        float4 y = x[pass];
-        y.x += o[pass].x; y.y += o[pass].y; y.z += o[pass].z; y.w += o[pass].w;
-        reinterpret_cast<float4*>(d[pass])[j] = y;
-        if (xb[pass])
-          *reinterpret_cast<uint2*>(xb[pass] + 4 * j) =
-              make_uint2(pack_bf16x2(y.x, y.y), pack_bf16x2(y.z, y.w));
-      }
-    } else {
-#pragma unroll
-      for (int pass = 0; pass < 8; ++pass) {
-        if (!d[pass]) continue;
-        float* q = reinterpret_cast<float*>(d[pass]) + 4 * j;
-        const float4 y = x[pass];
-        if (mode == EPI_GATE_RES)
-          red_add_v4(q, y.x, y.y, y.z, y.w);
-        else
-          *reinterpret_cast<float4*>(q) = y;
-      }
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                       s0 + lane * 64 + 16 * (j ^ ((lane >> 1) & 3))),
-                   "r"(pack_bf16x2(v[8 * j + 0], v[8 * j + 1])),
-                   "r"(pack_bf16x2(v[8 * j + 2], v[8 * j + 3])),
-                   "r"(pack_bf16x2(v[8 * j + 4], v[8 * j + 5])),
-                   "r"(pack_bf16x2(v[8 * j + 6], v[8 * j + 7]))
-                   : "memory");
-    __syncwarp();
-    const int j = lane & 3;
-    char* d[4];
-    uint4 x[4];
-#pragma unroll
-    for (int pass = 0; pass < 4; ++pass) {
-      const int row = pass * 8 + (lane >> 2);
-      d[pass] = reinterpret_cast<char*>(
-          __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), row));
-      x[pass] = *reinterpret_cast<const uint4*>(stg + row * 64 + 16 * (j ^ ((row >> 1) & 3)));
-    }
-#pragma unroll
-    for (int pass = 0; pass < 4; ++pass)
-      if (d[pass]) reinterpret_cast<uint4*>(d[pass])[j] = x[pass];
+  for (int pass = 0; pass < 8; ++pass) {
+    const int row = pass * 4 + (lane >> 3);
+    float* d = reinterpret_cast<float*>(
+        __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), row));
+    const float4 x = *reinterpret_cast<const float4*>(stg + row * 128 + 16 * (j ^ (row & 7)));
+    if (d) red_add_v4(d + 4 * j, x.x, x.y, x.z, x.w);
   }
   __syncwarp();  // the staging area is rewritten by the next chunk
+}
+
+// One warp's 32 x 32 chunk: lane = output row r (token tok, item item), v its
+// accumulator columns c0 .. c0 + 31 (cl within the tile).  x0: the row's
+// residual columns, loaded before the accumulator was ready (CAST).
+template <int MODE>
+__device__ __forceinline__ void finish_chunk(const GemmEpi& ep, int r, int M, int tok, int item,
+                                             int c0, int cl, float* v, const float* sv,
+                                             uint8_t* stg, int lane, const float* x0) {
+  epilogue_values<MODE>(ep, c0, cl, item, v, sv);
+  if (MODE == EPI_GATE_RES) {
+    reduce_chunk(stg, lane, v, r < M ? ep.xf + size_t(r) * ep.ld_xf + c0 : nullptr);
+    return;
+  }
+  if (r >= M) return;
+  if (MODE == EPI_F32) {  // (a caller's matrix: 16-byte aligned)
+    float4* d = reinterpret_cast<float4*>(ep.out_f + size_t(r) * ep.ld_out + c0);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+  } else if (MODE == EPI_GATE_RES_CAST) {
+    float* x = ep.xf + size_t(r) * ep.ld_xf + c0;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] += x0[i];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) st_v8(x + 8 * q, reinterpret_cast<const uint32_t*>(v + 8 * q));
+    store_bf16(ep.out_bf + size_t(r) * ep.ld_out + c0, v);
+  } else if (MODE == EPI_QKV) {
+    const int part = c0 / ep.dsplit, cc = c0 - part * ep.dsplit;
+    if (part == 0) {
+      store_bf16(ep.out_bf + size_t(r) * ep.ld_out + cc, v);
+    } else if (tok < 0 || tok >= ep.n_tokens || item < 0 || item >= ep.its.n) {
+      atomicOr(ep.err, DEVERR_INDEX);
+    } else {
+      store_bf16(ep.its.slice[item] + (part == 1 ? ep.k_off : ep.v_off) +
+                     size_t(tok) * ep.dsplit + cc,
+                 v);
+    }
+  } else {
+    store_bf16(ep.out_bf + size_t(r) * ep.ld_out + c0, v);
+  }
 }
 
 // Schedule, identical in every thread.  Tiles t = nn * mt + m (m fastest, so
@@ -401,9 +322,9 @@ struct Sched {
   // plus its exposed epilogues (~20 B/clk per SM with twelve epilogue warps;
   // all rates measured); a stream-K CTA holds two pieces.
   __host__ __device__ float cost(int out_bytes) const {
-    // one thread issues a tcgen05.mma about every 140 cycles (4 per k-block),
-    // two together twice as fast (one work item per CTA, tiles up to 192)
-    const float cmma = (alias && !pair && BN <= 192) ? 280.f : 560.f;
+    // the issuing thread takes about 290 cycles a k-block, the tensor pipe 4 MMAs
+    // of BN / 2 cycles
+    const float cmma = fmaxf(290.f, 2.f * float(BN) + 25.f);
     const float ckb = fmaxf(float(stage_bytes(BN, pair)) * (1.f / 60.f), cmma);
     const float cep = float(BM * BN * out_bytes) * (1.f / 20.f);
     if (S > 0) return float((kbt + S - 1) / S) * ckb + cep;
@@ -438,12 +359,12 @@ struct Sched {
     }
     return code;
   }
-  // table: the host's pick for 1 .. BN_TABLE row tiles (0 = not tabulated)
+  // table: the host's pick for 1 .. BN_TABLE row tiles
   __device__ void init(int M, int n, int k, int grid, int mode, const uint8_t* table, bool pr) {
     const int m_tiles = (M + BM - 1) / BM;
-    int code = m_tiles >= 1 && m_tiles <= BN_TABLE ? int(table[m_tiles - 1]) : 0;
-    if (code == 0) code = pick(M, n, k, grid, mode, pr);
-    plan(M, 64 * (code & 7), n, k, grid, mode == EPI_GATE_RES, code >> 3, pr);
+    const int code = int(table[m_tiles < 1 ? 0 : m_tiles <= BN_TABLE ? m_tiles - 1 : BN_TABLE - 1]);
+    plan(M, 64 * (code & 7), n, k, grid, mode == EPI_GATE_RES,
+         m_tiles <= BN_TABLE ? code >> 3 : 0, pr);
   }
   __device__ long long bound(int c) const { return Wr * c / Gr; }
 };
@@ -497,7 +418,7 @@ struct Segs {
 // 16 KB + BN x 64 B instead of 16 KB + BN x 128 B, so the ring keeps more
 // k-blocks in flight -- the main loop is bound by k-blocks in flight per SM
 // over the load latency.
-template <bool PAIR>
+template <int MODE, bool PAIR>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ BMaps tmB,
                int Mbound, const int* __restrict__ dcount, int n, int k,
@@ -515,7 +436,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * MAX_STAGES + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t full0 = saddr(bars), empty0 = saddr(bars + MAX_STAGES);
   const uint32_t tfull0 = saddr(bars + 2 * MAX_STAGES), tempty0 = saddr(bars + 2 * MAX_STAGES + 2);
 
@@ -540,7 +461,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     else
       tmem_alloc(saddr(tmem_slot), TMEM_COLS);
   }
-  if (warp == 0 && lane == 0)
+  if (warp == 0 && elect_one())
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
   tc_fence_before();
   __syncthreads();
@@ -554,37 +475,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // or more launches earlier (a step's dirty count before its first block;
   // every kernel of the library waits for its predecessor before letting its
   // successor start), so it and the schedule come before the programmatic-
-  // dependency wait; the operands and the residual are read after it
+  // dependency wait; the operand rows and the residual are read after it, by
+  // the warps that need them.  W is not the predecessor's either where the
+  // caller says so (ep.early_w)
   const int M = live_count(dcount, Mbound, ep.err);
   Sched sc;
   sc.init(M, n, k, int(gridDim.x), sched_mode(ep), bt.w64, PAIR);
-  pdl_wait();
-  pdl_trigger();
   const int BN = sc.BN, STAGES = sc.stages;
   const int STAGE = Sched::stage_bytes(BN, PAIR);
-  // split2: when every CTA holds one work item (so the second accumulator is
-  // free), two MMA threads take the item's even and odd k-blocks into the two
-  // accumulators, which the epilogue adds.  One thread issues a tcgen05.mma
-  // only about every 140 cycles when the ring stage is known at run time,
-  // whatever N; two threads together issue about twice as fast (measured).
-  // It shortens the main loop where few rows leave it bound by that issue
-  // rate (a sparse step at 5 % dirty: 397 -> 428 steps/s).  A 256-wide MMA
-  // keeps the tensor pipe busy about as long as one thread takes to issue
-  // it, so 256-wide tiles keep one issuer (the second accumulator's read in
-  // the epilogue would cost more than it saves: 298.7 -> 301.8 steps/s at
-  // 20 % dirty without it there).
-  const bool split2 = !PAIR && sc.alias && sc.kbt >= 2 && BN <= 192;
   // schedule position: the pair (its row tiles 2p + rank) or the CTA
   const int pos = PAIR ? int(blockIdx.x) >> 1 : int(blockIdx.x);
 
   if (warp == 0) {
     // ------------------------------------------------------- TMA producer
-    if (lane == 0) {
+    pdl_wait();
+    pdl_trigger();
+    if (elect_one()) {
       // W as one box of BN rows, or BN / 2 rows per CTA of a pair (maps for
       // the heights that divide n)
       const int brows = PAIR ? BN / 2 : BN;
       const CUtensorMap* tmW = &tmB.m[bmap_index(brows)];
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmW)) : "memory");
       int stage = 0;
       uint32_t phase = 0;
       Segs sg;
@@ -615,9 +525,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   } else if (warp == W_WARP) {
     // ------------------------------------------------------- TMA: W (unpaired)
-    if (!PAIR && lane == 0) {
+    if (!PAIR && elect_one()) {
       const CUtensorMap* tmW = &tmB.m[bmap_index(BN)];
-      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmW)) : "memory");
+      if (!ep.early_w) pdl_wait();
       int stage = 0;
       uint32_t phase = 0;
       Segs sg;
@@ -635,22 +545,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
-    if (lane == 0 && rank == 0 && split2) {
-      Segs sg;
-      sg.init(sc, pos);
-      int t, kb0, kb1;
-      if (sg.next(t, kb0, kb1) &&
-          !mma_half(0, kb0, kb1, STAGES, STAGE, saddr(smem), tmem_base,
-                    IDESC_BASE | (uint32_t(BN >> 3) << 17), full0, empty0, tfull0, tempty0,
-                    abort_flag))
-        goto timeout;
-    } else if (lane == 0 && rank == 0) {
+    if (rank == 0 && elect_one()) {
       const uint32_t idesc = (PAIR ? IDESC_PAIR : IDESC_BASE) | (uint32_t(BN >> 3) << 17);
       const uint64_t da = sw128_desc(saddr(smem)), db = sw128_desc(saddr(smem + STAGE_A));
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t acc_phase = 0;
+      bool ready = false;  // the current stage was seen full already
       Segs sg;
       sg.init(sc, pos);
       int t, kb0, kb1;
@@ -659,25 +561,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         tc_fence_after();
         const uint32_t dtm = tmem_base + uint32_t(acc * 256);
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) goto timeout;
-          tc_fence_after();
+          if (!ready && !mbar_wait(full0 + 8 * stage, phase, abort_flag)) goto timeout;
           // stage descriptors differ only in the start address field
           // (address >> 4; no carry out of its 14 bits below 256 KB)
           const uint64_t so = uint64_t((stage * STAGE) >> 4);
+          const uint32_t eb = empty0 + 8 * stage;
+          if (++stage == STAGES) { stage = 0; phase ^= 1; }
+          // the next stage is tested before this one's MMAs are issued, so
+          // that the test's latency (54 cycles) runs beside them
+          ready = mbar_test(full0 + 8 * stage, phase);
+          tc_fence_after();
           if (PAIR) {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
               umma_bf16_pair(dtm, da + so + 2 * kk, db + so + 2 * kk, idesc,
                              (kb > kb0 || kk > 0) ? 1u : 0u);
-            umma_commit_pair(empty0 + 8 * stage);  // frees the stage in both CTAs
+            umma_commit_pair(eb);  // frees the stage in both CTAs
           } else {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
               umma_bf16(dtm, da + so + 2 * kk, db + so + 2 * kk, idesc,
                         (kb > kb0 || kk > 0) ? 1u : 0u);
-            umma_commit(empty0 + 8 * stage);
+            umma_commit(eb);
           }
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
         if (PAIR)
           umma_commit_pair(tfull0 + 8 * acc);
@@ -685,18 +591,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           umma_commit(tfull0 + 8 * acc);
         if (++acc == 2) { acc = 0; acc_phase ^= 1; }
       }
-    }
-  } else if (warp == MMA2_WARP) {
-    // ------------------------------------------------------- second MMA issuer
-    if (lane == 0 && split2) {
-      Segs sg;
-      sg.init(sc, pos);
-      int t, kb0, kb1;
-      if (sg.next(t, kb0, kb1) &&
-          !mma_half(1, kb0, kb1, STAGES, STAGE, saddr(smem), tmem_base,
-                    IDESC_BASE | (uint32_t(BN >> 3) << 17), full0, empty0, tfull0, tempty0,
-                    abort_flag))
-        goto timeout;
     }
   } else {
     // ------------------------------------------------------- epilogue (warps 2..13)
@@ -713,39 +607,44 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // after a failed wait (it then skips the rest of the work), so that no
     // warp is ever left waiting at one
     bool ok = true;
+    pdl_wait();
     while (sg.next(t, kb0, kb1)) {
       const int mq = t % sc.mt, nn = t / sc.mt;
       const int m = PAIR ? 2 * mq + int(rank) : mq;
       // everything that does not depend on the accumulator first, while the
-      // main loop runs: the row's token / item, the tile's column vectors
+      // main loop runs: the row's token / item, the tile's column vectors,
+      // the first chunk's residual
       const int row = sp * 32 + lane;
       const int r = m * BM + row;
       int tok = 0, item = 0;
       if (r < M) {
-        if (ep.mode == EPI_QKV) tok = ep.tok ? __ldg(ep.tok + r) : r;
+        if (MODE == EPI_QKV) tok = ep.tok ? __ldg(ep.tok + r) : r;
         if (ep.item) item = __ldg(ep.item + r);
       }
+      constexpr int XN = MODE == EPI_GATE_RES_CAST ? 32 : 1;
+      float x0[XN];
+      auto load_x = [&](int ch) {
+        if (MODE == EPI_GATE_RES_CAST && r < M)
+#pragma unroll
+          for (int q = 0; q < XN / 8; ++q)
+            ld_v8(ep.xf + size_t(r) * ep.ld_xf + nn * BN + ch * 32 + 8 * q, x0 + 8 * q);
+      };
+      const int ch0 = (warp - 2) >> 2;
+      if (ch0 < BN / 32) load_x(ch0);
       epi_sync();  // the previous tile's readers of sVec are done
-      stage_vectors(ep, nn * BN, BN, kb0 == 0, sVec, int(threadIdx.x) - 64);
+      stage_vectors<MODE>(ep, nn * BN, BN, kb0 == 0, sVec, int(threadIdx.x) - 64);
       epi_sync();
-      if (ok && !mbar_wait_warp(tfull0 + 8 * acc, acc_phase, abort_flag)) ok = false;
-      if (ok && split2 && !mbar_wait_warp(tfull0 + 8, 0, abort_flag)) ok = false;
+      if (ok && !mbar_sleep_warp(tfull0 + 8 * acc, acc_phase, abort_flag)) ok = false;
       if (ok) {
         tc_fence_after();
         const uint32_t tbase = tmem_base + uint32_t(acc * 256) + (uint32_t(sp * 32) << 16);
 #pragma unroll 1
-        for (int ch = (warp - 2) >> 2; ch < BN / 32; ch += 3) {
+        for (int ch = ch0; ch < BN / 32; ch += 3) {
           float v[32];
-          if (split2)
-            tmem_ld32_sum2(tbase + uint32_t(ch * 32), v);
-          else
-            tmem_ld32(tbase + uint32_t(ch * 32), v);
-          const int c0 = nn * BN + ch * 32;
-          epilogue_values(ep, c0, ch * 32, item, v, sVec);
-          bf16* xb_row = (ep.mode == EPI_GATE_RES_CAST && r < M)
-                             ? ep.out_bf + size_t(r) * ep.ld_out + c0 : nullptr;
-          store_chunk(ep.mode, sStg + (warp - 2) * STAGING_WARP, lane, v,
-                      chunk_dst(ep, r, M, tok, item, c0), xb_row);
+          tmem_ld32(tbase + uint32_t(ch * 32), v);
+          if (ch != ch0) load_x(ch);
+          finish_chunk<MODE>(ep, r, M, tok, item, nn * BN + ch * 32, ch * 32, v, sVec,
+                             sStg + (warp - 2) * STAGING_WARP, lane, x0);
         }
         tc_fence_before();
         __syncwarp();
@@ -779,6 +678,20 @@ done:
       tmem_dealloc(tmem_base, TMEM_COLS);
   }
 }
+
+using GemmKernel = decltype(&gemm_tc_kernel<EPI_F32, false>);
+template <bool PAIR>
+GemmKernel gemm_kernel(int mode) {
+  switch (mode) {
+    case EPI_F32: return gemm_tc_kernel<EPI_F32, PAIR>;
+    case EPI_BIAS_BF16: return gemm_tc_kernel<EPI_BIAS_BF16, PAIR>;
+    case EPI_GELU_BF16: return gemm_tc_kernel<EPI_GELU_BF16, PAIR>;
+    case EPI_GATE_RES: return gemm_tc_kernel<EPI_GATE_RES, PAIR>;
+    case EPI_QKV: return gemm_tc_kernel<EPI_QKV, PAIR>;
+    default: return gemm_tc_kernel<EPI_GATE_RES_CAST, PAIR>;
+  }
+}
+constexpr int GEMM_MODES = 6;
 
 // ------------------------------------------------------------------- host
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -846,19 +759,20 @@ BnTable bn_table(int n, int k, int grid, int mode, int mt_bound, bool pair) {
   static std::mutex mu;
   static std::unordered_map<uint64_t, BnTable> cache;
   const int mtb = mt_bound < BN_TABLE ? mt_bound : BN_TABLE;
-  // bits: mtb 0-6, mode 7-9, pair 10, grid 11-18, k 19-40, n 41-63
+  // bits: mode 0-2, pair 3, grid 4-11, mtb 12-19, k 20-41, n 42-63
   // (mode < 8, grid < 256, n, k < 2^22: checked by the launcher)
-  const uint64_t full_key = uint64_t(mtb) | (uint64_t(mode & 7) << 7) |
-                            (uint64_t(pair ? 1 : 0) << 10) | (uint64_t(grid & 255) << 11) |
-                            (uint64_t(k & 0x3FFFFF) << 19) | (uint64_t(n) << 41);
+  const uint64_t full_key = uint64_t(mode & 7) | (uint64_t(pair ? 1 : 0) << 3) |
+                            (uint64_t(grid & 255) << 4) | (uint64_t(mtb) << 12) |
+                            (uint64_t(k & 0x3FFFFF) << 20) | (uint64_t(n) << 42);
   {
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(full_key);
     if (it != cache.end()) return it->second;
   }
   BnTable bt{};
-  for (int mt = 1; mt <= mtb; ++mt)
-    bt.w64[mt - 1] = uint8_t(Sched::pick(mt * BM, n, k, grid, mode, pair));
+  for (int mt = 1; mt <= BN_TABLE; ++mt)
+    bt.w64[mt - 1] =
+        mt <= mtb ? uint8_t(Sched::pick(mt * BM, n, k, grid, mode, pair)) : bt.w64[mt - 2];
   std::lock_guard<std::mutex> lock(mu);
   if (cache.size() > 4096) cache.clear();
   cache.emplace(full_key, bt);
@@ -891,11 +805,12 @@ GemmShape device_shape() {
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         v >= 256)
       return GemmShape{0, false};
-    if (cudaFuncSetAttribute(gemm_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(SMEM_BYTES)) != cudaSuccess ||
-        cudaFuncSetAttribute(gemm_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(SMEM_BYTES)) != cudaSuccess)
-      return GemmShape{0, false};
+    for (int mode = 0; mode < GEMM_MODES; ++mode)
+      if (cudaFuncSetAttribute(gemm_kernel<false>(mode), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(SMEM_BYTES)) != cudaSuccess ||
+          cudaFuncSetAttribute(gemm_kernel<true>(mode), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(SMEM_BYTES)) != cudaSuccess)
+        return GemmShape{0, false};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(v & ~1);
     cfg.blockDim = dim3(THREADS);
@@ -908,7 +823,7 @@ GemmShape device_shape() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, gemm_tc_kernel<true>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&nc, gemm_kernel<true>(EPI_F32), &cfg) != cudaSuccess) {
       cudaGetLastError();
       nc = 0;
     }
@@ -922,7 +837,8 @@ GemmShape device_shape() {
 cudaError_t launch_gemm(const bf16* A, int lda, const bf16* W, int Mbound, const int* dcount,
                         int n, int k, const GemmEpi& ep, cudaStream_t st) {
   if (Mbound <= 0) return cudaSuccess;
-  if (n % 64 || k % BK || n >= (1 << 22) || k >= (1 << 22) || ep.mode < 0 || ep.mode > 7)
+  if (n % 64 || k % BK || n >= (1 << 22) || k >= (1 << 22) || ep.mode < 0 ||
+      ep.mode >= GEMM_MODES)
     return cudaErrorInvalidValue;
   const GemmShape shp = device_shape();
   if (!shp.grid) return cudaErrorInvalidDevice;
@@ -945,10 +861,10 @@ cudaError_t launch_gemm(const bf16* A, int lda, const bf16* W, int Mbound, const
   const int grid = pair ? shp.grid : device_sms();
   const BnTable bt = bn_table(n, k, grid, sched_mode(ep), (Mbound + BM - 1) / BM, pair);
   if (pair)
-    RC_TRY(launch_k_cluster(gemm_tc_kernel<true>, dim3(shp.grid), dim3(THREADS), SMEM_BYTES, 2,
+    RC_TRY(launch_k_cluster(gemm_kernel<true>(ep.mode), dim3(shp.grid), dim3(THREADS), SMEM_BYTES, 2,
                             st, ta, tb, Mbound, dcount, n, k, ep, bt));
   else
-    RC_TRY(launch_k(gemm_tc_kernel<false>, dim3(grid), dim3(THREADS), SMEM_BYTES, st, ta, tb,
+    RC_TRY(launch_k(gemm_kernel<false>(ep.mode), dim3(grid), dim3(THREADS), SMEM_BYTES, st, ta, tb,
                     Mbound, dcount, n, k, ep, bt));
   count_launches(1);
   return cudaSuccess;

@@ -145,6 +145,7 @@ struct GemmEpi {
   unsigned* err;
   Items its;               // per-item cache slices and modulation vectors
   int whole_tiles;         // GATE_RES: no k split (one reduction per element, reproducible)
+  int early_w;             // W was complete before the preceding launch began
 };
 
 // C[M][n] = A[M][k] W[n][k]^T, epilogue `ep`.  M = *dcount if non-null (bounded

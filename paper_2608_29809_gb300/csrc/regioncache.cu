@@ -312,7 +312,10 @@ rc_status run_block(rc_ctx* c, rc_cache* k, int l, const rc::RowMap& rm, const S
   }
   if (h_stored) RC_CUDA(cudaEventRecord(h_stored, st), "H stored");
   // [q | k | v] = x_hat W_qkv^T + b; k, v rows go straight to cache rows tok[r]
+  // (the weights were complete long before any of the block's kernels: each
+  // is at least the second launch of its entry point)
   rc::GemmEpi e{};
+  e.early_w = 1;
   e.mode = rc::EPI_QKV;
   e.bias = w.b_qkv;
   e.out_bf = c->q;
@@ -343,6 +346,7 @@ rc_status run_block(rc_ctx* c, rc_cache* k, int l, const rc::RowMap& rm, const S
   // x += gate_msa (o W_o^T + b_o)
   auto gated = [&](const float* bias, int gate_k) {
     rc::GemmEpi g{};
+    g.early_w = 1;
     g.mode = rc::EPI_GATE_RES;
     g.bias = bias;
     g.xf = c->xf;
@@ -390,6 +394,7 @@ rc_status run_block(rc_ctx* c, rc_cache* k, int l, const rc::RowMap& rm, const S
   } else {
     // q' = x W_xq^T + b (on the bf16 copy of x)
     e = rc::GemmEpi{};
+    e.early_w = 1;
     e.mode = rc::EPI_BIAS_BF16;
     e.bias = w.b_xq;
     e.out_bf = c->q;
@@ -421,6 +426,7 @@ rc_status run_block(rc_ctx* c, rc_cache* k, int l, const rc::RowMap& rm, const S
             "ln_mod(mlp)");
   }
   e = rc::GemmEpi{};
+  e.early_w = 1;
   e.mode = rc::EPI_GELU_BF16;
   e.bias = w.b_1;
   e.out_bf = c->u;
