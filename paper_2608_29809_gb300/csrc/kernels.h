@@ -86,9 +86,11 @@ cudaError_t launch_batch_rows(const BatchIn& in, int* tok, int* item, int* meta,
 // ([6][d] vectors; tab may be null).  With hprev_off >= 0 the row itself is
 // also stored as bf16 to the item's cache slice at element offset
 // hprev_off + tok[r] * d (the previous block's merged hidden state, Section 3.3).
-cudaError_t launch_ln_mod(const float* x, const float* tab, int k_sh, int k_sc, const Items& it,
-                          bf16* out, const RowMap& rm, long long hprev_off, int d, unsigned* err,
-                          cudaStream_t st);
+// x_copy (null: x holds the compact rows): the rows are x[tok[r]] of the
+// caller's [N][d] matrix and are also copied to x_copy[r].
+cudaError_t launch_ln_mod(const float* x, float* x_copy, const float* tab, int k_sh, int k_sc,
+                          const Items& it, bf16* out, const RowMap& rm, long long hprev_off, int d,
+                          unsigned* err, cudaStream_t st);
 
 // xf[r] = W_e patch(tok[r]) + b_e + pos[tok[r]], the patch from the row's item latent.
 cudaError_t launch_patch_embed(int gh, int gw, int p, int C, const bf16* We, const float* be,
@@ -107,12 +109,9 @@ cudaError_t launch_final_ddim(const bf16* H, const float* temb, const float* tab
                               int p, int c_in, int c_out, int d, float ab_t, float ab_next,
                               cudaStream_t st);
 
-// dst[r] = src[idx[r]] (gather) or dst[idx[r]] = src[r] (scatter), f32 rows of d.
-cudaError_t launch_rows_f32(const float* src, float* dst, const int* idx, int Dbound,
-                            const int* dcount, int d, int N, bool scatter, unsigned* err,
-                            cudaStream_t st);
-// item slice + off + tok[r] * d  <-  bf16(src[r]), f32 rows -> bf16 cache rows.
-cudaError_t launch_scatter_bf16(const float* src, const Items& it, long long off,
+// item slice + off + tok[r] * d  <-  bf16(src[r]), f32 rows -> bf16 cache rows;
+// dst[tok[r]] <- src[r] too (f32 [N][d]; null: not).
+cudaError_t launch_scatter_bf16(const float* src, const Items& it, long long off, float* dst,
                                 const RowMap& rm, int d, unsigned* err, cudaStream_t st);
 
 // ---------------------------------------------------------------------- GEMM

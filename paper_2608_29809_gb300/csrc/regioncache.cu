@@ -295,10 +295,12 @@ rc::AttnItems text_kv_rows(const rc_cache* k, const StepItems& si, int l) {
 // vector of a row is tab (+ the row item's tb), each [6][d].  hprev_off >= 0:
 // the block input (the previous block's merged output H^l) is also written to
 // the cache slice at that element offset, and h_stored (if any) is recorded
-// on st once it is there.
+// on st once it is there.  With hidden the block's input rows are
+// hidden[tok[r]] ([N][d]) and c->xf is only written.
 rc_status run_block(rc_ctx* c, rc_cache* k, int l, const rc::RowMap& rm, const StepItems& si,
                     const float* tab, long long hprev_off, cudaStream_t st,
-                    const rc::AttnCapture* cap = nullptr, cudaEvent_t h_stored = nullptr) {
+                    const rc::AttnCapture* cap = nullptr, cudaEvent_t h_stored = nullptr,
+                    const float* hidden = nullptr) {
   const int d = c->d, F = c->F, N = c->N;
   const rc_layer_weights& w = c->lw[l];
   const size_t Nd = size_t(N) * d;
@@ -307,7 +309,8 @@ rc_status run_block(rc_ctx* c, rc_cache* k, int l, const rc::RowMap& rm, const S
   // block's output H^l of the dirty rows, written to their cache rows here
   {
     Probe pr(c, RC_PROBE_LN, st);
-    RC_CUDA(rc::launch_ln_mod(c->xf, tab, 0, 1, si.its, c->xb, rm, hprev_off, d, c->err, st),
+    RC_CUDA(rc::launch_ln_mod(hidden ? hidden : c->xf, hidden ? c->xf : nullptr, tab, 0, 1, si.its,
+                              c->xb, rm, hprev_off, d, c->err, st),
             "ln_mod(msa)");
   }
   if (h_stored) RC_CUDA(cudaEventRecord(h_stored, st), "H stored");
@@ -422,7 +425,7 @@ rc_status run_block(rc_ctx* c, rc_cache* k, int l, const rc::RowMap& rm, const S
   // MLP
   {
     Probe pr(c, RC_PROBE_LN, st);
-    RC_CUDA(rc::launch_ln_mod(c->xf, tab, 3, 4, si.its, c->xb, rm, -1, d, c->err, st),
+    RC_CUDA(rc::launch_ln_mod(c->xf, nullptr, tab, 3, 4, si.its, c->xb, rm, -1, d, c->err, st),
             "ln_mod(mlp)");
   }
   e = rc::GemmEpi{};
@@ -984,13 +987,11 @@ rc_status rc_block_forward_region(rc_ctx* c, rc_cache* k, int s, int l, int t, f
   si.session[0] = s;
   si.t[0] = t;
   const rc::RowMap rm{dirty_idx, nullptr, nullptr, bound, dirty_count, c->N};
-  RC_CUDA(rc::launch_rows_f32(hidden, c->xf, dirty_idx, bound, dirty_count, c->d, c->N, false,
-                              c->err, st), "gather");
-  if ((r = run_block(c, k, l, rm, si, mod6, -1, st))) return r;
-  RC_CUDA(rc::launch_scatter_bf16(c->xf, si.its, (long long)(size_t(l) * 3) * c->N * c->d, rm,
-                                  c->d, c->err, st), "H scatter");
-  RC_CUDA(rc::launch_rows_f32(c->xf, hidden, dirty_idx, bound, dirty_count, c->d, c->N, true,
-                              c->err, st), "scatter");
+  // the block's first LayerNorm gathers the dirty rows; its outputs go to the
+  // cache's H rows and back to `hidden` together
+  if ((r = run_block(c, k, l, rm, si, mod6, -1, st, nullptr, nullptr, hidden))) return r;
+  RC_CUDA(rc::launch_scatter_bf16(c->xf, si.its, (long long)(size_t(l) * 3) * c->N * c->d, hidden,
+                                  rm, c->d, c->err, st), "H scatter");
   return RC_OK;
 }
 
@@ -1156,8 +1157,8 @@ static rc_status step_items(rc_ctx* c, rc_cache* k, const rc_batch_item* items, 
       if (l > 0 && (r = host_writeback(c, k, s0, t0, l - 1, rm, st, false))) return r;
       if (l + 2 < L && (r = host_load(k, s0, t0, l + 2))) return r;
     }
-    RC_CUDA(rc::launch_scatter_bf16(c->xf, si.its, (long long)(size_t(L - 1) * 3) * Nd, rm, d,
-                                    c->err, st), "H scatter");
+    RC_CUDA(rc::launch_scatter_bf16(c->xf, si.its, (long long)(size_t(L - 1) * 3) * Nd, nullptr, rm,
+                                    d, c->err, st), "H scatter");
     if (host) {
       rc_status r = host_writeback(c, k, s0, t0, L - 1, rm, st, true);
       if (r) return r;
@@ -1379,7 +1380,7 @@ rc_status rc_localize_scores(rc_ctx* c, rc_cache* k, int s, int t, const float* 
   rc::Items cast{};
   cast.n = 1;
   cast.slice[0] = c->xb;
-  RC_CUDA(rc::launch_scatter_bf16(c->xf, cast, 0, rm, d, c->err, st), "embedding cast");
+  RC_CUDA(rc::launch_scatter_bf16(c->xf, cast, 0, nullptr, rm, d, c->err, st), "embedding cast");
   if (k->xg) {
     // (x W_xq^T + b) K^T = x G_h^T + kb_h with the folded text keys, every
     // layer in one launch (the layers' inputs are all in the cache)

@@ -367,11 +367,16 @@ cudaError_t launch_localize(const float* A, int S, int N, int M, int gh, int gw,
 }
 
 // ================================================================= LN + mod
-// One warp per row; the row stays in registers (hidden <= 1536, % 128 == 0).
-constexpr int LN_WARPS = 8;
-constexpr int LN_MAXV = 12;  // float4 per lane
-constexpr int LN_SV = (LN_MAXV * 32 + LN_WARPS * 32 - 1) / (LN_WARPS * 32);  // float4 per thread
-                                                                            // and staged vector
+// Four warps per row, at most three float4 of it per thread (hidden <= 1536,
+// % 128 == 0), so that a row is one short chain: its loads, two reductions
+// through shared memory, its stores.  A thread owns the same columns of every
+// row, so the shift and scale stay in its registers.  Bound by that chain at
+// small row counts (831 rows: 3 us after the dependency wait, as with a warp
+// per row) and by memory at large ones, where two CTAs an SM and the next
+// row's loads under this one's reductions count: 4096 rows 14.1 -> about 8 us.
+constexpr int LN_GROUP = 128, LN_ROWS = 4, LN_THREADS = LN_GROUP * LN_ROWS;
+constexpr int LN_V = 3;              // float4 per thread
+constexpr int LN_MAXD = LN_V * LN_GROUP * 4;
 
 // False (and DEVERR_INDEX) when a row's token or item is out of range.
 __device__ __forceinline__ bool row_valid(const RowMap& rm, int n_items, int tok, int item,
@@ -392,130 +397,146 @@ __device__ __forceinline__ bool row_target(const RowMap& rm, int n_items, int r,
   return row_valid(rm, n_items, tok, item, err, lane);
 }
 
-__global__ void __launch_bounds__(LN_WARPS * 32)
-ln_mod_kernel(const float* __restrict__ x, const float* __restrict__ tab, int k_sh, int k_sc,
+// Sum over the 128 threads of a row's group (red: 4 floats of the group's own
+// per call in flight).
+__device__ __forceinline__ float group_sum(float v, float* red, int group) {
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) & 3] = v;
+  // (constant barrier numbers: with one taken from a register a kernel
+  // reserves all sixteen)
+  static_assert(LN_ROWS == 4, "one barrier per row group");
+  if (group == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+  else if (group == 1) asm volatile("bar.sync 2, 128;" ::: "memory");
+  else if (group == 2) asm volatile("bar.sync 3, 128;" ::: "memory");
+  else asm volatile("bar.sync 4, 128;" ::: "memory");
+  return (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+__global__ void __launch_bounds__(LN_THREADS, 2)
+ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
+              const float* __restrict__ tab, int k_sh, int k_sc,
               const __grid_constant__ Items it, bf16* __restrict__ out, RowMap rm,
               long long hprev_off, int d, unsigned* err) {
-  // shift and scale staged once per CTA: tab (+ the item's tb when the
-  // launch has one item; otherwise each row adds its item's tb).  Loads that
-  // do not depend on one another are all issued before any is used (the
-  // vectors and the live row count, then the row with its token and item),
-  // so a CTA waits for about two L2 round trips before its arithmetic.
-  // The vectors and the row count are requested before the programmatic-
-  // dependency wait: this kernel is never the first of a step or a block
-  // call, and every kernel here waits for its predecessor before letting its
-  // successor start, so whatever was written two or more launches earlier
-  // (the modulation table and timestep vector, the dirty count) is complete
-  // when this kernel starts; only the rows x come from the predecessor.
-  extern __shared__ __align__(16) float s_mod[];  // [2][d]
-  const int lane = threadIdx.x & 31;
-  const int nv = d / 128, nq = d / 4;
+  // The shift / scale vectors and the row count are requested before the
+  // programmatic-dependency wait: every kernel here waits for its predecessor
+  // before letting its successor start, so whatever was written two or more
+  // launches earlier (the modulation table and timestep vector, the dirty
+  // count) is complete when this kernel starts; only the rows x come from the
+  // predecessor.  With x_copy the kernel is the first of its entry point and
+  // everything it reads is the caller's
+  __shared__ float s_red[LN_ROWS][2][4];
+  const int group = threadIdx.x / LN_GROUP, t = threadIdx.x % LN_GROUP, nq = d / 4;
+  if (x_copy) pdl_wait();
   const float* tb0 = it.n == 1 ? it.tb[0] : nullptr;
-  float4 m[4][LN_SV];  // tab shift, tab scale, tb shift, tb scale
+  float4 sh[LN_V], sc[LN_V];
+  {
+    float4 m[4][LN_V];  // tab shift, tab scale, tb shift, tb scale
 #pragma unroll
-  for (int j = 0; j < LN_SV; ++j) {
-    const int q = threadIdx.x + j * LN_WARPS * 32;
+    for (int j = 0; j < LN_V; ++j) {
+      const int q = t + j * LN_GROUP;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) m[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (q < nq && tab) {
-      m[0][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sh) * d) + q);
-      m[1][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sc) * d) + q);
+      for (int u = 0; u < 4; ++u) m[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (q < nq && tab) {
+        m[0][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sh) * d) + q);
+        m[1][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sc) * d) + q);
+      }
+      if (q < nq && tb0) {
+        m[2][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sh) * d) + q);
+        m[3][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sc) * d) + q);
+      }
     }
-    if (q < nq && tb0) {
-      m[2][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sh) * d) + q);
-      m[3][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sc) * d) + q);
+#pragma unroll
+    for (int j = 0; j < LN_V; ++j) {
+      sh[j] = make_float4(m[0][j].x + m[2][j].x, m[0][j].y + m[2][j].y, m[0][j].z + m[2][j].z,
+                          m[0][j].w + m[2][j].w);
+      sc[j] = make_float4(m[1][j].x + m[3][j].x, m[1][j].y + m[3][j].y, m[1][j].z + m[3][j].z,
+                          m[1][j].w + m[3][j].w);
     }
   }
   const int D = live_count(rm.count, rm.bound, err);
   pdl_wait();
   pdl_trigger();
-  int r = blockIdx.x * LN_WARPS + (threadIdx.x >> 5);
-  float4 v[LN_MAXV];
+  int r = blockIdx.x * LN_ROWS + group;
+  float4 v[LN_V];
   int tok = 0, item = 0;
+  bool ok = false;
   auto load_row = [&](int rr) {
     tok = rm.tok ? __ldg(rm.tok + rr) : rr;
     item = rm.item ? __ldg(rm.item + rr) : 0;
-    const float4* xr = reinterpret_cast<const float4*>(x + size_t(rr) * d);
+    if (x_copy) ok = row_valid(rm, it.n, tok, item, err, t);
+    const float4* xr = reinterpret_cast<const float4*>(x + size_t(x_copy ? (ok ? tok : 0) : rr) * d);
 #pragma unroll
-    for (int k = 0; k < LN_MAXV; ++k)
-      if (k < nv) v[k] = xr[lane + 32 * k];
+    for (int j = 0; j < LN_V; ++j)
+      v[j] = t + j * LN_GROUP < nq ? xr[t + j * LN_GROUP] : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!x_copy) ok = row_valid(rm, it.n, tok, item, err, t);
   };
   if (r < D) load_row(r);
-#pragma unroll
-  for (int j = 0; j < LN_SV; ++j) {
-    const int q = threadIdx.x + j * LN_WARPS * 32;
-    if (q < nq) {
-      float4 a = m[0][j], b = m[1][j];
-      if (tb0) {
-        a.x += m[2][j].x; a.y += m[2][j].y; a.z += m[2][j].z; a.w += m[2][j].w;
-        b.x += m[3][j].x; b.y += m[3][j].y; b.z += m[3][j].z; b.w += m[3][j].w;
-      }
-      reinterpret_cast<float4*>(s_mod)[q] = a;
-      reinterpret_cast<float4*>(s_mod + d)[q] = b;
-    }
-  }
-  __syncthreads();
   while (r < D) {
-    if (row_valid(rm, it.n, tok, item, err, lane)) {
-      float s = 0.f;
+    float4 y[LN_V];
 #pragma unroll
-      for (int k = 0; k < LN_MAXV; ++k)
-        if (k < nv) s += (v[k].x + v[k].y) + (v[k].z + v[k].w);
-      if (hprev_off >= 0) {
-        uint2* hrow = reinterpret_cast<uint2*>(it.slice[item] + hprev_off + size_t(tok) * d);
+    for (int j = 0; j < LN_V; ++j) y[j] = v[j];
+    const int row = r, rtok = tok, ritem = item;
+    const bool rok = ok;
+    r += gridDim.x * LN_ROWS;
+    if (r < D) load_row(r);  // the group's next row, under this one's reductions
+    if (!rok) continue;      // (the same for the whole group)
+    float s = 0.f;
 #pragma unroll
-        for (int k = 0; k < LN_MAXV; ++k)
-          if (k < nv)
-            hrow[lane + 32 * k] =
-                make_uint2(pack_bf16x2(v[k].x, v[k].y), pack_bf16x2(v[k].z, v[k].w));
-      }
-      const float mean = warp_sum(s) / float(d);
-      float q = 0.f;
+    for (int j = 0; j < LN_V; ++j) s += (y[j].x + y[j].y) + (y[j].z + y[j].w);
+    if (hprev_off >= 0) {
+      uint2* hrow = reinterpret_cast<uint2*>(it.slice[ritem] + hprev_off + size_t(rtok) * d);
 #pragma unroll
-      for (int k = 0; k < LN_MAXV; ++k)
-        if (k < nv) {
-          float a = v[k].x - mean, b = v[k].y - mean, c = v[k].z - mean, e = v[k].w - mean;
-          q += (a * a + b * b) + (c * c + e * e);
-        }
-      const float rstd = 1.0f / sqrtf(warp_sum(q) / float(d) + 1e-6f);
-      const float* tb = tb0 ? nullptr : it.tb[item];
-      uint2* orow = reinterpret_cast<uint2*>(out + size_t(r) * d);
-#pragma unroll
-      for (int k = 0; k < LN_MAXV; ++k)
-        if (k < nv) {
-          const int c = 4 * (lane + 32 * k);
-          float4 sh = *reinterpret_cast<const float4*>(s_mod + c);
-          float4 sc = *reinterpret_cast<const float4*>(s_mod + d + c);
-          if (tb) {
-            const float4 a = *reinterpret_cast<const float4*>(tb + size_t(k_sh) * d + c);
-            const float4 b = *reinterpret_cast<const float4*>(tb + size_t(k_sc) * d + c);
-            sh.x += a.x; sh.y += a.y; sh.z += a.z; sh.w += a.w;
-            sc.x += b.x; sc.y += b.y; sc.z += b.z; sc.w += b.w;
-          }
-          float y0 = (v[k].x - mean) * rstd * (1.f + sc.x) + sh.x;
-          float y1 = (v[k].y - mean) * rstd * (1.f + sc.y) + sh.y;
-          float y2 = (v[k].z - mean) * rstd * (1.f + sc.z) + sh.z;
-          float y3 = (v[k].w - mean) * rstd * (1.f + sc.w) + sh.w;
-          orow[lane + 32 * k] = make_uint2(pack_bf16x2(y0, y1), pack_bf16x2(y2, y3));
-        }
+      for (int j = 0; j < LN_V; ++j)
+        if (t + j * LN_GROUP < nq)
+          hrow[t + j * LN_GROUP] =
+              make_uint2(pack_bf16x2(y[j].x, y[j].y), pack_bf16x2(y[j].z, y[j].w));
     }
-    r += gridDim.x * LN_WARPS;
-    if (r < D) load_row(r);
+    if (x_copy) {
+      float4* c = reinterpret_cast<float4*>(x_copy + size_t(row) * d);
+#pragma unroll
+      for (int j = 0; j < LN_V; ++j)
+        if (t + j * LN_GROUP < nq) c[t + j * LN_GROUP] = y[j];
+    }
+    const float mean = group_sum(s, s_red[group][0], group) / float(d);
+    float q = 0.f;
+#pragma unroll
+    for (int j = 0; j < LN_V; ++j)
+      if (t + j * LN_GROUP < nq) {
+        y[j].x -= mean; y[j].y -= mean; y[j].z -= mean; y[j].w -= mean;
+        q += (y[j].x * y[j].x + y[j].y * y[j].y) + (y[j].z * y[j].z + y[j].w * y[j].w);
+      }
+    const float rstd = 1.0f / sqrtf(group_sum(q, s_red[group][1], group) / float(d) + 1e-6f);
+    const float* tb = tb0 ? nullptr : it.tb[ritem];
+    uint2* orow = reinterpret_cast<uint2*>(out + size_t(row) * d);
+#pragma unroll
+    for (int j = 0; j < LN_V; ++j)
+      if (t + j * LN_GROUP < nq) {
+        float4 a = sh[j], b = sc[j];
+        if (tb) {
+          const float4* tq = reinterpret_cast<const float4*>(tb) + t + j * LN_GROUP;
+          const float4 ta = __ldg(tq + size_t(k_sh) * nq), sb = __ldg(tq + size_t(k_sc) * nq);
+          a.x += ta.x; a.y += ta.y; a.z += ta.z; a.w += ta.w;
+          b.x += sb.x; b.y += sb.y; b.z += sb.z; b.w += sb.w;
+        }
+        const float y0 = y[j].x * rstd * (1.f + b.x) + a.x;
+        const float y1 = y[j].y * rstd * (1.f + b.y) + a.y;
+        const float y2 = y[j].z * rstd * (1.f + b.z) + a.z;
+        const float y3 = y[j].w * rstd * (1.f + b.w) + a.w;
+        orow[t + j * LN_GROUP] = make_uint2(pack_bf16x2(y0, y1), pack_bf16x2(y2, y3));
+      }
   }
 }
 
-cudaError_t launch_ln_mod(const float* x, const float* tab, int k_sh, int k_sc, const Items& it,
-                          bf16* out, const RowMap& rm, long long hprev_off, int d, unsigned* err,
-                          cudaStream_t st) {
+cudaError_t launch_ln_mod(const float* x, float* x_copy, const float* tab, int k_sh, int k_sc,
+                          const Items& it, bf16* out, const RowMap& rm, long long hprev_off, int d,
+                          unsigned* err, cudaStream_t st) {
   if (rm.bound <= 0) return cudaSuccess;
-  if (d % 128 || d > 128 * LN_MAXV) return cudaErrorInvalidValue;
-  RC_TRY(launch_k(ln_mod_kernel, dim3(row_grid(rm.bound, LN_WARPS, 1)), dim3(LN_WARPS * 32),
-                  size_t(2) * d * sizeof(float), st, x, tab, k_sh, k_sc, it, out, rm, hprev_off,
-                  d, err));
+  if (d % 128 || d > LN_MAXD) return cudaErrorInvalidValue;
+  RC_TRY(launch_k(ln_mod_kernel, dim3(row_grid(rm.bound, LN_ROWS, 2)), dim3(LN_THREADS), 0, st, x,
+                  x_copy, tab, k_sh, k_sc, it, out, rm, hprev_off, d, err));
   count_launches(1);
   return cudaSuccess;
 }
-
 
 // ============================================================ patch embed
 // x_r = W_e patch(idx[r]) + b_e + pos[idx[r]], the patch vector ordered
@@ -883,33 +904,14 @@ cudaError_t launch_final_ddim(const bf16* H, const float* temb, const float* tab
   return cudaSuccess;
 }
 
-// ======================================================= gather / scatter
-// One warp per row, grid-stride over the rows.
+// ================================================================== scatter
+// One warp per row, grid-stride over the rows; the rows also go to dst (f32,
+// null: not) at their tokens.
 constexpr int RW_WARPS = 8;
 
 __global__ void __launch_bounds__(RW_WARPS * 32)
-rows_f32_kernel(const float* __restrict__ src, float* __restrict__ dst,
-                const int* __restrict__ idx, int Dbound, const int* __restrict__ dcount, int d,
-                int N, int scatter, unsigned* err) {
-  pdl_wait();
-  pdl_trigger();
-  const int D = live_count(dcount, Dbound, err);
-  const int lane = threadIdx.x & 31;
-  for (int r = blockIdx.x * RW_WARPS + (threadIdx.x >> 5); r < D; r += gridDim.x * RW_WARPS) {
-    const int i = idx[r];
-    if (i < 0 || i >= N) {
-      if (lane == 0) atomicOr(err, DEVERR_INDEX);
-      continue;
-    }
-    const float4* s4 = reinterpret_cast<const float4*>(src + size_t(scatter ? r : i) * d);
-    float4* t4 = reinterpret_cast<float4*>(dst + size_t(scatter ? i : r) * d);
-    for (int c = lane; c < d / 4; c += 32) t4[c] = s4[c];
-  }
-}
-
-__global__ void __launch_bounds__(RW_WARPS * 32)
 scatter_bf16_kernel(const float* __restrict__ src, const __grid_constant__ Items it,
-                    long long off, RowMap rm, int d, unsigned* err) {
+                    long long off, float* __restrict__ dst, RowMap rm, int d, unsigned* err) {
   pdl_wait();
   pdl_trigger();
   const int D = live_count(rm.count, rm.bound, err);
@@ -919,9 +921,19 @@ scatter_bf16_kernel(const float* __restrict__ src, const __grid_constant__ Items
     if (!row_target(rm, it.n, r, i, item, err, lane)) continue;
     const float4* s4 = reinterpret_cast<const float4*>(src + size_t(r) * d);
     uint2* t2 = reinterpret_cast<uint2*>(it.slice[item] + off + size_t(i) * d);
-    for (int c = lane; c < d / 4; c += 32) {
-      const float4 v = s4[c];
-      t2[c] = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+    float4* f4 = reinterpret_cast<float4*>(dst + size_t(i) * d);
+    constexpr int B = 6;  // loads in flight
+    for (int c0 = lane; c0 < d / 4; c0 += 32 * B) {
+      float4 v[B];
+#pragma unroll
+      for (int e = 0; e < B; ++e)
+        if (c0 + 32 * e < d / 4) v[e] = s4[c0 + 32 * e];
+#pragma unroll
+      for (int e = 0; e < B; ++e)
+        if (c0 + 32 * e < d / 4) {
+          t2[c0 + 32 * e] = make_uint2(pack_bf16x2(v[e].x, v[e].y), pack_bf16x2(v[e].z, v[e].w));
+          if (dst) f4[c0 + 32 * e] = v[e];
+        }
     }
   }
 }
@@ -1015,21 +1027,11 @@ cudaError_t launch_batch_rows(const BatchIn& in, int* tok, int* item, int* meta,
   return cudaSuccess;
 }
 
-cudaError_t launch_rows_f32(const float* src, float* dst, const int* idx, int Dbound,
-                            const int* dcount, int d, int N, bool scatter, unsigned* err,
-                            cudaStream_t st) {
-  if (Dbound <= 0) return cudaSuccess;
-  RC_TRY(launch_k(rows_f32_kernel, dim3(row_grid(Dbound, RW_WARPS, 4)), dim3(RW_WARPS * 32), 0, st,
-                  src, dst, idx, Dbound, dcount, d, N, scatter ? 1 : 0, err));
-  count_launches(1);
-  return cudaSuccess;
-}
-
-cudaError_t launch_scatter_bf16(const float* src, const Items& it, long long off,
+cudaError_t launch_scatter_bf16(const float* src, const Items& it, long long off, float* dst,
                                 const RowMap& rm, int d, unsigned* err, cudaStream_t st) {
   if (rm.bound <= 0) return cudaSuccess;
-  RC_TRY(launch_k(scatter_bf16_kernel, dim3(row_grid(rm.bound, RW_WARPS, 1)), dim3(RW_WARPS * 32),
-                  0, st, src, it, off, rm, d, err));
+  RC_TRY(launch_k(scatter_bf16_kernel, dim3(row_grid(rm.bound, RW_WARPS, 4)), dim3(RW_WARPS * 32),
+                  0, st, src, it, off, dst, rm, d, err));
   count_launches(1);
   return cudaSuccess;
 }
