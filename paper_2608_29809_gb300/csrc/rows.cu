@@ -367,16 +367,17 @@ cudaError_t launch_localize(const float* A, int S, int N, int M, int gh, int gw,
 }
 
 // ================================================================= LN + mod
-// Four warps per row, at most three float4 of it per thread (hidden <= 1536,
-// % 128 == 0), so that a row is one short chain: its loads, two reductions
-// through shared memory, its stores.  A thread owns the same columns of every
-// row, so the shift and scale stay in its registers.  Bound by that chain at
-// small row counts (831 rows: 3 us after the dependency wait, as with a warp
-// per row) and by memory at large ones, where two CTAs an SM and the next
-// row's loads under this one's reductions count: 4096 rows 14.1 -> about 8 us.
-constexpr int LN_GROUP = 128, LN_ROWS = 4, LN_THREADS = LN_GROUP * LN_ROWS;
-constexpr int LN_V = 3;              // float4 per thread
-constexpr int LN_MAXD = LN_V * LN_GROUP * 4;
+// One warp per row; the row stays in registers (hidden <= 1536, % 128 == 0).
+// Bound by the row's chain of latencies at small row counts, by issue slots
+// and memory at large ones: three CTAs of eight warps an SM take 3648 rows at
+// once, and consecutive rows go to different CTAs, so that few rows spread
+// over the whole chip.  (Four warps per row halve a row's chain but double its
+// instructions: 4096 rows took 13.5 us that way, 8.3 this way; 831 rows 4.9
+// and 3.7.)
+constexpr int LN_WARPS = 8, LN_CTAS = 3;
+constexpr int LN_MAXV = 12;  // float4 per lane
+constexpr int LN_SV = (LN_MAXV * 32 + LN_WARPS * 32 - 1) / (LN_WARPS * 32);  // float4 per thread
+                                                                            // and staged vector
 
 // False (and DEVERR_INDEX) when a row's token or item is out of range.
 __device__ __forceinline__ bool row_valid(const RowMap& rm, int n_items, int tok, int item,
@@ -397,132 +398,111 @@ __device__ __forceinline__ bool row_target(const RowMap& rm, int n_items, int r,
   return row_valid(rm, n_items, tok, item, err, lane);
 }
 
-// Sum over the 128 threads of a row's group (red: 4 floats of the group's own
-// per call in flight).
-__device__ __forceinline__ float group_sum(float v, float* red, int group) {
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) red[(threadIdx.x >> 5) & 3] = v;
-  // (constant barrier numbers: with one taken from a register a kernel
-  // reserves all sixteen)
-  static_assert(LN_ROWS == 4, "one barrier per row group");
-  if (group == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
-  else if (group == 1) asm volatile("bar.sync 2, 128;" ::: "memory");
-  else if (group == 2) asm volatile("bar.sync 3, 128;" ::: "memory");
-  else asm volatile("bar.sync 4, 128;" ::: "memory");
-  return (red[0] + red[1]) + (red[2] + red[3]);
-}
-
-__global__ void __launch_bounds__(LN_THREADS, 2)
+__global__ void __launch_bounds__(LN_WARPS * 32, LN_CTAS)
 ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
               const float* __restrict__ tab, int k_sh, int k_sc,
               const __grid_constant__ Items it, bf16* __restrict__ out, RowMap rm,
               long long hprev_off, int d, unsigned* err) {
-  // The shift / scale vectors and the row count are requested before the
-  // programmatic-dependency wait: every kernel here waits for its predecessor
-  // before letting its successor start, so whatever was written two or more
-  // launches earlier (the modulation table and timestep vector, the dirty
-  // count) is complete when this kernel starts; only the rows x come from the
+  // shift and scale staged once per CTA: tab (+ the item's tb when the
+  // launch has one item; otherwise each row adds its item's tb).
+  // The vectors and the row count are requested before the programmatic-
+  // dependency wait: every kernel here waits for its predecessor before
+  // letting its successor start, so whatever was written two or more launches
+  // earlier (the modulation table and timestep vector, the dirty count) is
+  // complete when this kernel starts; only the rows x come from the
   // predecessor.  With x_copy the kernel is the first of its entry point and
   // everything it reads is the caller's
-  __shared__ float s_red[LN_ROWS][2][4];
-  const int group = threadIdx.x / LN_GROUP, t = threadIdx.x % LN_GROUP, nq = d / 4;
+  extern __shared__ __align__(16) float s_mod[];  // [2][d]
+  const int lane = threadIdx.x & 31;
+  const int nv = d / 128, nq = d / 4;
   if (x_copy) pdl_wait();
   const float* tb0 = it.n == 1 ? it.tb[0] : nullptr;
-  float4 sh[LN_V], sc[LN_V];
-  {
-    float4 m[4][LN_V];  // tab shift, tab scale, tb shift, tb scale
+  float4 m[4][LN_SV];  // tab shift, tab scale, tb shift, tb scale
 #pragma unroll
-    for (int j = 0; j < LN_V; ++j) {
-      const int q = t + j * LN_GROUP;
+  for (int j = 0; j < LN_SV; ++j) {
+    const int q = threadIdx.x + j * LN_WARPS * 32;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) m[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (q < nq && tab) {
-        m[0][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sh) * d) + q);
-        m[1][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sc) * d) + q);
-      }
-      if (q < nq && tb0) {
-        m[2][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sh) * d) + q);
-        m[3][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sc) * d) + q);
-      }
+    for (int u = 0; u < 4; ++u) m[u][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (q < nq && tab) {
+      m[0][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sh) * d) + q);
+      m[1][j] = __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sc) * d) + q);
     }
-#pragma unroll
-    for (int j = 0; j < LN_V; ++j) {
-      sh[j] = make_float4(m[0][j].x + m[2][j].x, m[0][j].y + m[2][j].y, m[0][j].z + m[2][j].z,
-                          m[0][j].w + m[2][j].w);
-      sc[j] = make_float4(m[1][j].x + m[3][j].x, m[1][j].y + m[3][j].y, m[1][j].z + m[3][j].z,
-                          m[1][j].w + m[3][j].w);
+    if (q < nq && tb0) {
+      m[2][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sh) * d) + q);
+      m[3][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sc) * d) + q);
     }
   }
   const int D = live_count(rm.count, rm.bound, err);
+#pragma unroll
+  for (int j = 0; j < LN_SV; ++j) {
+    const int q = threadIdx.x + j * LN_WARPS * 32;
+    if (q < nq) {
+      float4 a = m[0][j], b = m[1][j];
+      if (tb0) {
+        a.x += m[2][j].x; a.y += m[2][j].y; a.z += m[2][j].z; a.w += m[2][j].w;
+        b.x += m[3][j].x; b.y += m[3][j].y; b.z += m[3][j].z; b.w += m[3][j].w;
+      }
+      reinterpret_cast<float4*>(s_mod)[q] = a;
+      reinterpret_cast<float4*>(s_mod + d)[q] = b;
+    }
+  }
+  __syncthreads();
   pdl_wait();
   pdl_trigger();
-  int r = blockIdx.x * LN_ROWS + group;
-  float4 v[LN_V];
-  int tok = 0, item = 0;
-  bool ok = false;
-  auto load_row = [&](int rr) {
-    tok = rm.tok ? __ldg(rm.tok + rr) : rr;
-    item = rm.item ? __ldg(rm.item + rr) : 0;
-    if (x_copy) ok = row_valid(rm, it.n, tok, item, err, t);
-    const float4* xr = reinterpret_cast<const float4*>(x + size_t(x_copy ? (ok ? tok : 0) : rr) * d);
+  for (int r = blockIdx.x + gridDim.x * (threadIdx.x >> 5); r < D; r += gridDim.x * LN_WARPS) {
+    const int tok = rm.tok ? __ldg(rm.tok + r) : r;
+    const int item = rm.item ? __ldg(rm.item + r) : 0;
+    if (x_copy && !row_valid(rm, it.n, tok, item, err, lane)) continue;
+    const float4* xr = reinterpret_cast<const float4*>(x + size_t(x_copy ? tok : r) * d);
+    float4 v[LN_MAXV];
 #pragma unroll
-    for (int j = 0; j < LN_V; ++j)
-      v[j] = t + j * LN_GROUP < nq ? xr[t + j * LN_GROUP] : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!x_copy) ok = row_valid(rm, it.n, tok, item, err, t);
-  };
-  if (r < D) load_row(r);
-  while (r < D) {
-    float4 y[LN_V];
-#pragma unroll
-    for (int j = 0; j < LN_V; ++j) y[j] = v[j];
-    const int row = r, rtok = tok, ritem = item;
-    const bool rok = ok;
-    r += gridDim.x * LN_ROWS;
-    if (r < D) load_row(r);  // the group's next row, under this one's reductions
-    if (!rok) continue;      // (the same for the whole group)
+    for (int k = 0; k < LN_MAXV; ++k)
+      if (k < nv) v[k] = xr[lane + 32 * k];
+    if (!x_copy && !row_valid(rm, it.n, tok, item, err, lane)) continue;
     float s = 0.f;
 #pragma unroll
-    for (int j = 0; j < LN_V; ++j) s += (y[j].x + y[j].y) + (y[j].z + y[j].w);
+    for (int k = 0; k < LN_MAXV; ++k)
+      if (k < nv) s += (v[k].x + v[k].y) + (v[k].z + v[k].w);
     if (hprev_off >= 0) {
-      uint2* hrow = reinterpret_cast<uint2*>(it.slice[ritem] + hprev_off + size_t(rtok) * d);
+      uint2* hrow = reinterpret_cast<uint2*>(it.slice[item] + hprev_off + size_t(tok) * d);
 #pragma unroll
-      for (int j = 0; j < LN_V; ++j)
-        if (t + j * LN_GROUP < nq)
-          hrow[t + j * LN_GROUP] =
-              make_uint2(pack_bf16x2(y[j].x, y[j].y), pack_bf16x2(y[j].z, y[j].w));
+      for (int k = 0; k < LN_MAXV; ++k)
+        if (k < nv)
+          hrow[lane + 32 * k] =
+              make_uint2(pack_bf16x2(v[k].x, v[k].y), pack_bf16x2(v[k].z, v[k].w));
     }
     if (x_copy) {
-      float4* c = reinterpret_cast<float4*>(x_copy + size_t(row) * d);
+      float4* c = reinterpret_cast<float4*>(x_copy + size_t(r) * d);
 #pragma unroll
-      for (int j = 0; j < LN_V; ++j)
-        if (t + j * LN_GROUP < nq) c[t + j * LN_GROUP] = y[j];
+      for (int k = 0; k < LN_MAXV; ++k)
+        if (k < nv) c[lane + 32 * k] = v[k];
     }
-    const float mean = group_sum(s, s_red[group][0], group) / float(d);
+    const float mean = warp_sum(s) / float(d);
     float q = 0.f;
 #pragma unroll
-    for (int j = 0; j < LN_V; ++j)
-      if (t + j * LN_GROUP < nq) {
-        y[j].x -= mean; y[j].y -= mean; y[j].z -= mean; y[j].w -= mean;
-        q += (y[j].x * y[j].x + y[j].y * y[j].y) + (y[j].z * y[j].z + y[j].w * y[j].w);
+    for (int k = 0; k < LN_MAXV; ++k)
+      if (k < nv) {
+        v[k].x -= mean; v[k].y -= mean; v[k].z -= mean; v[k].w -= mean;
+        q += (v[k].x * v[k].x + v[k].y * v[k].y) + (v[k].z * v[k].z + v[k].w * v[k].w);
       }
-    const float rstd = 1.0f / sqrtf(group_sum(q, s_red[group][1], group) / float(d) + 1e-6f);
-    const float* tb = tb0 ? nullptr : it.tb[ritem];
-    uint2* orow = reinterpret_cast<uint2*>(out + size_t(row) * d);
+    const float rstd = 1.0f / sqrtf(warp_sum(q) / float(d) + 1e-6f);
+    const float* tb = tb0 ? nullptr : it.tb[item];
+    uint2* orow = reinterpret_cast<uint2*>(out + size_t(r) * d);
 #pragma unroll
-    for (int j = 0; j < LN_V; ++j)
-      if (t + j * LN_GROUP < nq) {
-        float4 a = sh[j], b = sc[j];
+    for (int k = 0; k < LN_MAXV; ++k)
+      if (k < nv) {
+        const int c = 4 * (lane + 32 * k);
+        float4 sh = *reinterpret_cast<const float4*>(s_mod + c);
+        float4 sc = *reinterpret_cast<const float4*>(s_mod + d + c);
         if (tb) {
-          const float4* tq = reinterpret_cast<const float4*>(tb) + t + j * LN_GROUP;
-          const float4 ta = __ldg(tq + size_t(k_sh) * nq), sb = __ldg(tq + size_t(k_sc) * nq);
-          a.x += ta.x; a.y += ta.y; a.z += ta.z; a.w += ta.w;
-          b.x += sb.x; b.y += sb.y; b.z += sb.z; b.w += sb.w;
+          const float4 a = __ldg(reinterpret_cast<const float4*>(tb + size_t(k_sh) * d + c));
+          const float4 b = __ldg(reinterpret_cast<const float4*>(tb + size_t(k_sc) * d + c));
+          sh.x += a.x; sh.y += a.y; sh.z += a.z; sh.w += a.w;
+          sc.x += b.x; sc.y += b.y; sc.z += b.z; sc.w += b.w;
         }
-        const float y0 = y[j].x * rstd * (1.f + b.x) + a.x;
-        const float y1 = y[j].y * rstd * (1.f + b.y) + a.y;
-        const float y2 = y[j].z * rstd * (1.f + b.z) + a.z;
-        const float y3 = y[j].w * rstd * (1.f + b.w) + a.w;
-        orow[t + j * LN_GROUP] = make_uint2(pack_bf16x2(y0, y1), pack_bf16x2(y2, y3));
+        orow[lane + 32 * k] = make_uint2(
+            pack_bf16x2(v[k].x * rstd * (1.f + sc.x) + sh.x, v[k].y * rstd * (1.f + sc.y) + sh.y),
+            pack_bf16x2(v[k].z * rstd * (1.f + sc.z) + sh.z, v[k].w * rstd * (1.f + sc.w) + sh.w));
       }
   }
 }
@@ -531,9 +511,10 @@ cudaError_t launch_ln_mod(const float* x, float* x_copy, const float* tab, int k
                           const Items& it, bf16* out, const RowMap& rm, long long hprev_off, int d,
                           unsigned* err, cudaStream_t st) {
   if (rm.bound <= 0) return cudaSuccess;
-  if (d % 128 || d > LN_MAXD) return cudaErrorInvalidValue;
-  RC_TRY(launch_k(ln_mod_kernel, dim3(row_grid(rm.bound, LN_ROWS, 2)), dim3(LN_THREADS), 0, st, x,
-                  x_copy, tab, k_sh, k_sc, it, out, rm, hprev_off, d, err));
+  if (d % 128 || d > 128 * LN_MAXV) return cudaErrorInvalidValue;
+  RC_TRY(launch_k(ln_mod_kernel, dim3(row_grid(rm.bound, 1, LN_CTAS)), dim3(LN_WARPS * 32),
+                  size_t(2) * d * sizeof(float), st, x, x_copy, tab, k_sh, k_sc, it, out, rm,
+                  hprev_off, d, err));
   count_launches(1);
   return cudaSuccess;
 }
