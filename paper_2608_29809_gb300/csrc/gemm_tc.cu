@@ -56,6 +56,8 @@ constexpr int THREADS = 480;
 constexpr int W_WARP = 14;
 constexpr int STAGE_A = BM * BK * 2;   // bytes
 constexpr int MIN_KB_PER_CTA = 4;
+// most equal parts of the k range of one tile (codes BN / 64 + 8 S are bytes)
+constexpr int MAX_SPLIT = 8;
 constexpr int STAGING_WARP = 32 * 128;  // epilogue staging: 32 rows of 128 B per warp
 constexpr int STAGING_BYTES = 12 * STAGING_WARP;
 
@@ -318,18 +320,21 @@ struct Sched {
     return s < MAX_STAGES ? s : MAX_STAGES;
   }
   // Estimated duration (SM cycles): k-blocks on the busiest CTA x per-k-block
-  // time (operands at ~60 B/clk per SM, but no less than the MMA issue time)
-  // plus its exposed epilogues (~20 B/clk per SM with twelve epilogue warps;
-  // all rates measured); a stream-K CTA holds two pieces.
-  __host__ __device__ float cost(int out_bytes) const {
-    // the issuing thread takes about 290 cycles a k-block, the tensor pipe 4 MMAs
-    // of BN / 2 cycles
-    const float cmma = fmaxf(290.f, 2.f * float(BN) + 25.f);
-    const float ckb = fmaxf(float(stage_bytes(BN, pair)) * (1.f / 60.f), cmma);
-    const float cep = float(BM * BN * out_bytes) * (1.f / 20.f);
+  // time plus its exposed epilogues; a stream-K CTA holds two pieces.  Rates
+  // measured on the five matrices of a 1152-wide block at 39 to 4096 rows:
+  // single CTAs take 220 / 365 / 435 / 540 cycles a k-block at BN 64 / 128 /
+  // 192 / 256, pairs 280 / 356 / 430 / 570 (operands at ~60 B/clk per SM, but
+  // no less than the MMA issue time); an epilogue drains ~20 B/clk per SM
+  // (15 where the output is reduced in place), and half of one shows on
+  // every further wave.
+  __host__ __device__ float cost(int out_bytes, bool additive) const {
+    const float ckb =
+        pair ? fmaxf(float(stage_bytes(BN, pair)) * (1.f / 60.f), 2.f * float(BN) + 25.f)
+             : 125.f + 1.65f * float(BN);
+    const float cep = float(BM * BN * out_bytes) * (additive ? 1.f / 15.f : 1.f / 20.f);
     if (S > 0) return float((kbt + S - 1) / S) * ckb + cep;
     const int waves = (whole + G - 1) / G;
-    float c = float(waves) * float(kbt) * ckb + (waves > 0 ? cep : 0.f);
+    float c = float(waves) * (float(kbt) * ckb + 0.5f * cep) + (waves > 0 ? 0.5f * cep : 0.f);
     if (Gr > 0) c += float((Wr + Gr - 1) / Gr) * ckb + 2.f * cep;
     return c;
   }
@@ -346,11 +351,11 @@ struct Sched {
     int code = 1;
     for (int i = 0; i < 4; ++i) {
       if (n % cand[i]) continue;
-      for (int sp = 0; sp <= (additive ? 4 : 0); ++sp) {
+      for (int sp = 0; sp <= (additive ? MAX_SPLIT : 0); ++sp) {
         if (sp == 1) continue;
         s.plan(M, cand[i], n, k, grid, additive, sp, pr);
         if (sp > 0 && (s.tiles * sp > s.G || s.kbt < sp * MIN_KB_PER_CTA)) continue;
-        const float c = s.cost(out_bytes);
+        const float c = s.cost(out_bytes, additive);
         if (c < best * 0.999f) {
           best = c;
           code = cand[i] / 64 + 8 * sp;
