@@ -92,10 +92,11 @@ cudaError_t launch_ln_mod(const float* x, float* x_copy, const float* tab, int k
                           const Items& it, bf16* out, const RowMap& rm, long long hprev_off, int d,
                           unsigned* err, cudaStream_t st);
 
-// xf[r] = W_e patch(tok[r]) + b_e + pos[tok[r]], the patch from the row's item latent.
+// xf[r] = W_e patch(tok[r]) + b_e + pos[tok[r]], the patch from the row's item
+// latent; with xb its bf16 rounding goes there instead (xf may be null).
 cudaError_t launch_patch_embed(int gh, int gw, int p, int C, const bf16* We, const float* be,
                                const float* pos, const Items& it, const RowMap& rm, float* xf,
-                               int d, unsigned* err, cudaStream_t st);
+                               bf16* xb, int d, unsigned* err, cudaStream_t st);
 
 // Timestep embedding chain: f = sinusoid(t_value); h1 = W_t1 f + b; temb = W_t2 silu(h1) + b;
 // tb = W_tb silu(temb) + b.  scratch h1/f are caller buffers.

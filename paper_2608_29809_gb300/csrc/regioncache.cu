@@ -1128,7 +1128,7 @@ static rc_status step_items(rc_ctx* c, rc_cache* k, const rc_batch_item* items, 
     }
     RC_CUDA(rc::launch_patch_embed(c->dims.grid_h, c->dims.grid_w, c->dims.patch, c->dims.in_ch,
                                    static_cast<const bf16*>(g.W_e), g.b_e, g.pos, si.its, rm,
-                                   c->xf, d, c->err, st),
+                                   c->xf, nullptr, d, c->err, st),
             "patch_embed");
     for (int l = 0; l < L; ++l) {
       if (!host) {
@@ -1368,19 +1368,15 @@ rc_status rc_localize_scores(rc_ctx* c, rc_cache* k, int s, int t, const float* 
   RC_CUDA(cudaMemsetAsync(scores, 0, sizeof(float) * size_t(N) * c->M, st), "scores reset");
   // every token is a query row, in token order
   const rc::RowMap rm{nullptr, nullptr, nullptr, N, nullptr, N};
-  // the state entering block 0: the patch embedding of the latent (f32),
-  // then its bf16 copy for the query side of the cross-attention
+  // the state entering block 0, in bf16 for the query side of the
+  // cross-attention: the patch embedding of the latent
   rc::Items its{};
   its.n = 1;
   its.latent[0] = const_cast<float*>(latent);
   RC_CUDA(rc::launch_patch_embed(c->dims.grid_h, c->dims.grid_w, c->dims.patch, c->dims.in_ch,
-                                 static_cast<const bf16*>(g.W_e), g.b_e, g.pos, its, rm, c->xf, d,
-                                 c->err, st),
+                                 static_cast<const bf16*>(g.W_e), g.b_e, g.pos, its, rm, nullptr,
+                                 c->xb, d, c->err, st),
           "patch_embed");
-  rc::Items cast{};
-  cast.n = 1;
-  cast.slice[0] = c->xb;
-  RC_CUDA(rc::launch_scatter_bf16(c->xf, cast, 0, nullptr, rm, d, c->err, st), "embedding cast");
   if (k->xg) {
     // (x W_xq^T + b) K^T = x G_h^T + kb_h with the folded text keys, every
     // layer in one launch (the layers' inputs are all in the cache)

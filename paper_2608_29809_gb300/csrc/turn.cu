@@ -332,50 +332,77 @@ fold_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUt
 
 // ------------------------------------------------- localisation scores
 // scores[i][j] = mean over layers and heads of softmax_j'((x_i G_h^T + kb_h)
-// / sqrt(dh))[j] for the listed columns j.  One persistent CTA an SM; a unit
-// is 128 tokens of one layer and two heads: S = x G^T with M = 128, N = 256
-// (the two heads' 128 key rows), k-blocks of 16 + 32 KB through a 4-stage
-// ring.  Bound by the tensor pipe (18 x 4 MMAs of 128 cycles a unit), so the
+// / sqrt(dh))[j] for the listed columns j.  Persistent, one CTA an SM; a unit
+// is one layer and two heads of a token tile: S = x G^T with the two heads' key
+// rows, each rounded up to 8, as N <= 256 columns.  Two token tiles share a
+// unit as a CTA pair (M = 256): a CTA then holds 16 + 16 KB a k-block instead of
+// 16 + 32, so 7 k-blocks are in flight instead of 4 over a load latency of
+// 1400 cycles and more.  Bound by the tensor pipe under the power cap, so the
 // two 256-column accumulators alternate and eight warps take the softmax of
-// one unit under the MMAs of the next.  Units are handed out in contiguous
-// ranges, tokens outermost: a thread keeps its token's sums over layers and
-// heads in registers and adds them to memory once per range and token tile.
-constexpr int SC_STAGES = 4, SC_THREADS = 384, SC_STAGE = A_TILE + 256 * 128;
-constexpr size_t SC_SMEM = size_t(SC_STAGES) * SC_STAGE + 1024;
+// one unit under the MMAs of the next.  4096 tokens x 28 layers x 16 heads x
+// 120 keys: 329 us with single CTAs and all 128 rows a head, 318 without the
+// rows past the text, 296 (1.7 PFLOP/s) in pairs.  Units are handed out in
+// contiguous ranges, tokens outermost: a thread keeps its token's sums over
+// layers and heads in registers and adds them to memory once per range and
+// token tile.
+constexpr int SC_THREADS = 384;
+// CTAs a unit, stages of the ring and bytes of one in a CTA
+template <int CL>
+struct ScoreCfg {
+  static constexpr int STAGES = CL == 2 ? 7 : 4;
+  static constexpr int STAGE = A_TILE + 2 / CL * XQ_KEYS * 128;
+  static constexpr size_t SMEM = size_t(STAGES) * STAGE + 1024;
+};
 constexpr int SC_MAX = 8;  // listed columns
 
+template <int CL>
 __global__ void __launch_bounds__(SC_THREADS, 1)
 scores_kernel(const __grid_constant__ CUtensorMap tmX0, const __grid_constant__ CUtensorMap tmX,
               const __grid_constant__ CUtensorMap tmG, const float* __restrict__ kb, int N, int d,
               int layers, int heads, int xrow0, int xrow_step, int grow0, int Nk,
               float scale_log2, const __grid_constant__ AttnCapture cap, unsigned* err) {
+  using C = ScoreCfg<CL>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  __shared__ uint64_t bars[2 * SC_STAGES + 4];
+  __shared__ uint64_t bars[2 * C::STAGES + 4];
   __shared__ uint32_t tmem_slot;
   __shared__ int s_abort;
   volatile int* abort_flag = &s_abort;
-  const uint32_t full0 = saddr(bars), empty0 = full0 + 8 * SC_STAGES;
-  const uint32_t t_full = empty0 + 8 * SC_STAGES, t_free = t_full + 16;
+  const uint32_t full0 = saddr(bars), empty0 = full0 + 8 * C::STAGES;
+  const uint32_t t_full = empty0 + 8 * C::STAGES, t_free = t_full + 16;
   const int warp = warp_index(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int i = 0; i < 2 * SC_STAGES + 2; ++i) mbar_init(full0 + 8 * i, 1);
-    mbar_init(t_free, 256);
-    mbar_init(t_free + 8, 256);
+    for (int i = 0; i < C::STAGES; ++i) {
+      mbar_init(full0 + 8 * i, 1);
+      mbar_init(empty0 + 8 * i, 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(t_full + 8 * i, 1);
+      mbar_init(t_free + 8 * i, 8 * CL);  // one arrival a softmax warp
+    }
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 1) tmem_alloc(saddr(&tmem_slot), 512);
+  if (warp == 1) {
+    if (CL == 2) tmem_alloc_pair(saddr(&tmem_slot), 512);
+    else tmem_alloc(saddr(&tmem_slot), 512);
+  }
   tc_fence_before();
-  __syncthreads();
+  if (CL == 2) cluster_sync();  // (the peer's barriers are set up)
+  else __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  const int rank = CL == 2 ? int(cluster_ctarank()) : 0;
   const int pairs = heads / 2, per_tile = layers * pairs, nkb = d / TK;
-  const long long units = (long long)((N + TM - 1) / TM) * per_tile;
-  const int u0 = int(units * blockIdx.x / gridDim.x), u1 = int(units * (blockIdx.x + 1) / gridDim.x);
+  const int keys = (Nk + 7) & ~7;  // rows of a head in a stage
+  const long long units = (long long)((N + CL * TM - 1) / (CL * TM)) * per_tile;
+  const int pos = int(blockIdx.x) / CL, np = int(gridDim.x) / CL;
+  const int u0 = int(units * pos / np), u1 = int(units * (pos + 1) / np);
   pdl_wait();
   pdl_trigger();
-  if (warp == 0) {
+  if (warp == 0 || warp == 2) {
+    // warp 0 loads the token rows, warp 2 the folded keys: one thread issuing
+    // both is close to the time of a k-block's MMAs
     if (elect_one()) {
       int st = 0;
       uint32_t ph = 1;
@@ -384,48 +411,78 @@ scores_kernel(const __grid_constant__ CUtensorMap tmX0, const __grid_constant__ 
         const int grow = grow0 + (l * heads + 2 * (rest - l * pairs)) * XQ_KEYS;
         // layer 0 reads the embedding, layer l the cached output of l - 1
         const CUtensorMap* mx = l ? &tmX : &tmX0;
-        const int xrow = qt * TM + (l ? xrow0 + (l - 1) * xrow_step : 0);
+        const int xrow = (qt * CL + rank) * TM + (l ? xrow0 + (l - 1) * xrow_step : 0);
         for (int k = 0; k < nkb; ++k) {
-          if (!mbar_sleep(empty0 + 8 * st, ph, abort_flag)) {
+          if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
             *abort_flag = 1;
             goto out;
           }
-          mbar_expect_tx(full0 + 8 * st, SC_STAGE);
-          uint8_t* b = smem + st * SC_STAGE;
-          tma_load_2d(saddr(b), mx, full0 + 8 * st, k * TK, xrow);
-          tma_load_2d(saddr(b + A_TILE), &tmG, full0 + 8 * st, k * TK, grow);
-          if (++st == SC_STAGES) { st = 0; ph ^= 1; }
+          uint8_t* b = smem + st * C::STAGE;
+          if (CL == 2) {  // all of a pair's bytes are counted by rank 0's barrier
+            const uint32_t fb = mapa_shared(full0 + 8 * st, 0);
+            if (warp == 2) {
+              tma_load_2d_pair(saddr(b + A_TILE), &tmG, fb, k * TK, grow + rank * XQ_KEYS);
+            } else {
+              if (rank == 0)
+                mbar_expect_tx(full0 + 8 * st, uint32_t(2 * (A_TILE + keys * 128)));
+              tma_load_2d_pair(saddr(b), mx, fb, k * TK, xrow);
+            }
+          } else if (warp == 2) {
+            for (int g = 0; g < 2; ++g)
+              tma_load_2d(saddr(b + A_TILE + g * keys * 128), &tmG, full0 + 8 * st, k * TK,
+                          grow + g * XQ_KEYS);
+          } else {
+            mbar_expect_tx(full0 + 8 * st, uint32_t(A_TILE + 2 * keys * 128));
+            tma_load_2d(saddr(b), mx, full0 + 8 * st, k * TK, xrow);
+          }
+          if (++st == C::STAGES) { st = 0; ph ^= 1; }
         }
+      }
+      // every stage has been freed: no arrival is on its way to this CTA when
+      // it leaves
+      for (int i = 0; CL == 2 && i < C::STAGES; ++i) {
+        if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) goto out;
+        if (++st == C::STAGES) { st = 0; ph ^= 1; }
       }
     }
   } else if (warp == 1) {
-    if (elect_one()) {
+    if (rank == 0 && elect_one()) {
       const uint64_t da = sw128_desc(saddr(smem)), db = sw128_desc(saddr(smem + A_TILE));
+      // (M = 256 over a pair: bits 24.. hold M / 16)
+      const uint32_t id = (idesc(0, false) + (CL == 2 ? uint32_t(TM >> 4) << 24 : 0u)) |
+                          (uint32_t(2 * keys) >> 3 << 17);
       int st = 0;
       uint32_t ph = 0;
+      bool ready = false;  // the current stage was seen full already
       for (int u = u0; u < u1; ++u) {
         const int i = u - u0;
-        if (!mbar_sleep(t_free + 8 * (i & 1), ((i >> 1) & 1) ^ 1, abort_flag)) {
+        if (!mbar_wait(t_free + 8 * (i & 1), ((i >> 1) & 1) ^ 1, abort_flag)) {
           *abort_flag = 1;
           goto out;
         }
         tc_fence_after();
         const uint32_t acc = tmem + 256u * uint32_t(i & 1);
         for (int k = 0; k < nkb; ++k) {
-          if (!mbar_sleep(full0 + 8 * st, ph, abort_flag)) {
+          if (!ready && !mbar_wait(full0 + 8 * st, ph, abort_flag)) {
             *abort_flag = 1;
             goto out;
           }
+          const uint64_t so = uint64_t((st * C::STAGE) >> 4);
+          const uint32_t eb = empty0 + 8 * st;
+          if (++st == C::STAGES) { st = 0; ph ^= 1; }
+          ready = mbar_test(full0 + 8 * st, ph);  // (beside this stage's MMAs)
           tc_fence_after();
-          const uint64_t so = uint64_t((st * SC_STAGE) >> 4);
 #pragma unroll
-          for (int kk = 0; kk < TK / 16; ++kk)
-            umma_bf16(acc, da + so + 2 * kk, db + so + 2 * kk, idesc(256, false),
-                      (k > 0 || kk > 0) ? 1u : 0u);
-          umma_commit(empty0 + 8 * st);
-          if (++st == SC_STAGES) { st = 0; ph ^= 1; }
+          for (int kk = 0; kk < TK / 16; ++kk) {
+            const uint32_t add = (k > 0 || kk > 0) ? 1u : 0u;
+            if (CL == 2) umma_bf16_pair(acc, da + so + 2 * kk, db + so + 2 * kk, id, add);
+            else umma_bf16(acc, da + so + 2 * kk, db + so + 2 * kk, id, add);
+          }
+          if (CL == 2) umma_commit_pair(eb);
+          else umma_commit(eb);
         }
-        umma_commit(t_full + 8 * (i & 1));
+        if (CL == 2) umma_commit_pair(t_full + 8 * (i & 1));
+        else umma_commit(t_full + 8 * (i & 1));
       }
     }
   } else if (warp >= 4) {
@@ -435,7 +492,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmX0, const __grid_constant__ 
     for (int q = 0; q < SC_MAX; ++q) acc[q] = 0.f;
     int qt = u0 / per_tile;
     auto flush = [&]() {
-      const int tok = qt * TM + sp * 32 + lane;
+      const int tok = (qt * CL + rank) * TM + sp * 32 + lane;
       if (tok < N) {
 #pragma unroll
         for (int q = 0; q < SC_MAX; ++q)
@@ -458,7 +515,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmX0, const __grid_constant__ 
       }
       tc_fence_after();
       const uint32_t ts =
-          tmem + 256u * uint32_t(i & 1) + 128u * uint32_t(half) + (uint32_t(sp * 32) << 16);
+          tmem + 256u * uint32_t(i & 1) + uint32_t(half * keys) + (uint32_t(sp * 32) << 16);
       const float* b = kb + size_t(grow0) + (size_t(l) * heads + h) * XQ_KEYS;
       float r[XQ_KEYS];
 #pragma unroll
@@ -492,17 +549,23 @@ scores_kernel(const __grid_constant__ CUtensorMap tmX0, const __grid_constant__ 
           acc[q] += ex2_ftz(fmaf(__uint_as_float(v) + __ldg(b + cap.id[q]), scale_log2, -m)) * inv;
         }
       tc_fence_before();
-      mbar_arrive(t_free + 8 * (i & 1));
+      __syncwarp();
+      if (lane == 0) {
+        if (CL == 2) mbar_arrive_cluster(mapa_shared(t_free + 8 * (i & 1), 0));
+        else mbar_arrive(t_free + 8 * (i & 1));
+      }
     }
     if (u1 > u0) flush();
   }
 out:
   tc_fence_before();
   __syncthreads();
+  if (CL == 2) cluster_sync();  // the peer's loads and arrivals in this CTA are done
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    if (CL == 2) tmem_dealloc_pair(tmem, 512);
+    else tmem_dealloc(tmem, 512);
   }
 }
 
@@ -517,7 +580,8 @@ int turn_sms() {
         cudaFuncSetAttribute(text_kv_kernel, attr, int(KV_SMEM)) != cudaSuccess ||
         cudaFuncSetAttribute(fold_kernel<72>, attr, int(FoldCfg<72>::SMEM)) != cudaSuccess ||
         cudaFuncSetAttribute(fold_kernel<64>, attr, int(FoldCfg<64>::SMEM)) != cudaSuccess ||
-        cudaFuncSetAttribute(scores_kernel, attr, int(SC_SMEM)) != cudaSuccess)
+        cudaFuncSetAttribute(scores_kernel<1>, attr, int(ScoreCfg<1>::SMEM)) != cudaSuccess ||
+        cudaFuncSetAttribute(scores_kernel<2>, attr, int(ScoreCfg<2>::SMEM)) != cudaSuccess)
       return 0;
     sms[dev] = v;
   }
@@ -625,12 +689,22 @@ cudaError_t launch_scores(const bf16* x0, int x0_rows, const bf16* cache, long l
   dims[1] = cuuint64_t(cache_rows);
   RC_TRY(tma_map(cache, 2, dims, str, box, &tx));
   dims[1] = cuuint64_t(g_rows);
-  box[1] = 2 * XQ_KEYS;
+  box[1] = cuuint32_t((Nk + 7) & ~7);
   RC_TRY(tma_map(G, 2, dims, str, box, &tg));
   const float scale_log2 = float(1.4426950408889634 / sqrt(double(dh)));
-  const int grid = int(units < sms ? units : sms);
-  RC_TRY(launch_k(scores_kernel, dim3(grid), dim3(SC_THREADS), SC_SMEM, st, t0, tx, tg, kb, N, d,
-                  layers, heads, xrow0, xrow_step, grow0, Nk, scale_log2, cap, err));
+  // pairs wherever there are two token tiles (a single one would leave half of
+  // each pair idle)
+  if (N > TM && sms >= 2) {
+    const long long pairs = (long long)((N + 2 * TM - 1) / (2 * TM)) * layers * (heads / 2);
+    const int grid = 2 * int(pairs < sms / 2 ? pairs : sms / 2);
+    RC_TRY(launch_k_cluster(scores_kernel<2>, dim3(grid), dim3(SC_THREADS),
+                            ScoreCfg<2>::SMEM, 2, st, t0, tx, tg, kb, N, d, layers, heads, xrow0, xrow_step, grow0, Nk,
+                            scale_log2, cap, err));
+  } else {
+    const int grid = int(units < sms ? units : sms);
+    RC_TRY(launch_k(scores_kernel<1>, dim3(grid), dim3(SC_THREADS), ScoreCfg<1>::SMEM, st,
+                    t0, tx, tg, kb, N, d, layers, heads, xrow0, xrow_step, grow0, Nk, scale_log2, cap, err));
+  }
   count_launches(1);
   return cudaSuccess;
 }
