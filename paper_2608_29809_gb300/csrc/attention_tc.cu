@@ -1012,12 +1012,10 @@ xattn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // One (query tile, head) per CTA: S = xb_tile G_h^T accumulated over d in
 // 64-column k-blocks (TMA ring, M = 128, N = 128), then the softmax of
 // (S + kb) / sqrt(dh) per row, P over S in TMEM, O = P V, O / l stored.
-// Two threads issue the S MMAs, the even k-blocks into S0 and the odd ones
-// into S1 (TMEM columns 0 / 128; the softmax adds them): one thread issues
-// a tcgen05.mma only about every 140 cycles from a ring whose stage is known
-// at run time, and the 72 MMAs of the d = 1152 loop were bound by that.
+// One warp loads the keys and V (from before the dependency wait on), one the
+// rows, one issues the MMAs with the next stage tested ahead.
 constexpr int XF_STAGES = 6;
-constexpr int XF_THREADS = 224;  // TMA, MMA, 4 softmax warps, second MMA warp
+constexpr int XF_THREADS = 224;  // rows, MMA, 4 softmax warps, keys and V
 template <int DH>
 struct XFCfg {
   using C = ACfg<DH>;
@@ -1051,14 +1049,14 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   const uint32_t full0 = saddr(bars), empty0 = saddr(bars + XF_STAGES);
   const uint32_t v_full = saddr(bars + 2 * XF_STAGES), s_full = v_full + 8, p_ready = v_full + 16,
                  o_full = v_full + 24, kb_ready = v_full + 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < XF_STAGES; ++i) {
       mbar_init(full0 + 8 * i, 1);
       mbar_init(empty0 + 8 * i, 1);
     }
     mbar_init(v_full, 1);
-    mbar_init(s_full, 2);  // both MMA threads commit their half of S
+    mbar_init(s_full, 1);
     mbar_init(p_ready, 128);
     mbar_init(o_full, 1);
     mbar_init(kb_ready, 128);
@@ -1076,73 +1074,77 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   // the grid covers the bound of the query tiles: CTAs past the live ones
   // leave at once, before taking tensor memory
   if (qt >= qtiles) return;
-  const bool live = true;
   const TileLoc tl = locate_tile(rm, xi.n, D, qt);
-  // one CTA per SM (its shared memory), so all 512 columns are there
-  if (warp == 1) tmem_alloc(saddr(tmem_slot), 512);
+  if (warp == 1) tmem_alloc(saddr(tmem_slot), 256);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // S0 | S1 | O; P is written over S0
-  const uint32_t tS = tmem_base, tS1 = tmem_base + XK, tO = tmem_base + 2 * XK;
+  // S | O; P is written over S
+  const uint32_t tS = tmem_base, tO = tmem_base + XK;
   const int nkb = d / 64;
-  bool ok = live;
-  if (live && warp == 0 && lane == 0) {
-    // ------------------------------------------------------------ TMA
-    // V and the folded keys of the first stages before the wait (each stage
-    // barrier expects both halves of its bytes), the x rows after it
-    const int grow = xi.grow[tl.item] + h * XK;
-    mbar_expect_tx(v_full, X::V_BYTES);
-    tma_load_3d(saddr(sV), &tmV, v_full, 0, h, xi.vrow[tl.item]);
-    if (C::TAIL) tma_load_3d(saddr(sV + X::V_ATOM), &tmV, v_full, 64, h, xi.vrow[tl.item]);
-    const int pre = nkb < XF_STAGES ? nkb : XF_STAGES;
-    for (int k = 0; k < pre; ++k) {
-      mbar_expect_tx(full0 + 8 * k, X::STAGE);
-      tma_load_3d(saddr(smem + k * X::STAGE + X::STAGE_A), &tmG, full0 + 8 * k, 0, k, grow);
-    }
+  bool ok = true;
+  if (warp == 0) {
+    // ------------------------------------------------------------ TMA: rows
     pdl_wait();
     pdl_trigger();
-    for (int k = 0; k < nkb; ++k) {
-      const int st = k % XF_STAGES;
-      uint8_t* base = smem + st * X::STAGE;
-      if (k >= pre) {
-        if (!mbar_wait(empty0 + 8 * st, ((k / XF_STAGES) & 1) ^ 1, abort_flag)) {
+    if (elect_one()) {
+      int st = 0;
+      uint32_t ph = 1;
+      for (int k = 0; k < nkb; ++k) {
+        if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
           *abort_flag = 1;
           break;
         }
+        // (the keys may arrive before this expectation: the phase still
+        // needs this arrival)
         mbar_expect_tx(full0 + 8 * st, X::STAGE);
-        tma_load_3d(saddr(base + X::STAGE_A), &tmG, full0 + 8 * st, 0, k, grow);
+        tma_load_3d(saddr(smem + st * X::STAGE), &tmA, full0 + 8 * st, 0, k, tl.row0);
+        if (++st == XF_STAGES) { st = 0; ph ^= 1; }
       }
-      tma_load_3d(saddr(base), &tmA, full0 + 8 * st, 0, k, tl.row0);
     }
-  } else if (live && (warp == 1 || warp == 6) && lane == 0) {
+  } else if (warp == 6) {
+    // ------------------------------------------------------------ TMA: keys, V
+    if (elect_one()) {
+      const int grow = xi.grow[tl.item] + h * XK;
+      int st = 0;
+      uint32_t ph = 1;
+      for (int k = 0; k < nkb; ++k) {
+        if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
+          *abort_flag = 1;
+          break;
+        }
+        tma_load_3d(saddr(smem + st * X::STAGE + X::STAGE_A), &tmG, full0 + 8 * st, 0, k, grow);
+        if (++st == XF_STAGES) { st = 0; ph ^= 1; }
+        if (k == (nkb < XF_STAGES ? nkb : XF_STAGES) - 1) {  // the ring is filled: V
+          mbar_expect_tx(v_full, X::V_BYTES);
+          tma_load_3d(saddr(sV), &tmV, v_full, 0, h, xi.vrow[tl.item]);
+          if (C::TAIL) tma_load_3d(saddr(sV + X::V_ATOM), &tmV, v_full, 64, h, xi.vrow[tl.item]);
+        }
+      }
+    }
+  } else if (warp == 1 && elect_one()) {
     // ------------------------------------------------------------ MMA
-    // warp 1: the even k-blocks into S0, then P V; warp 6: the odd ones into S1
-    pdl_wait();
-    const int par = warp == 1 ? 0 : 1;
-    const uint32_t dS = par ? tS1 : tS;
     const uint64_t da = sw128_desc(saddr(smem)), dg = sw128_desc(saddr(smem + X::STAGE_A));
-    bool good = true;
-    for (int k = par; k < nkb && good; k += 2) {
-      const int st = k % XF_STAGES;
-      if (!mbar_wait(full0 + 8 * st, (k / XF_STAGES) & 1, abort_flag)) {
+    bool good = true, ready = false;
+    int st = 0;
+    uint32_t ph = 0;
+    for (int k = 0; k < nkb; ++k) {
+      if (!ready && !mbar_wait(full0 + 8 * st, ph, abort_flag)) {
         good = false;
         break;
       }
-      tc_fence_after();
       const uint64_t so = uint64_t((st * X::STAGE) >> 4);
+      const uint32_t eb = empty0 + 8 * st;
+      if (++st == XF_STAGES) { st = 0; ph ^= 1; }
+      ready = mbar_test(full0 + 8 * st, ph);  // (beside this stage's MMAs)
+      tc_fence_after();
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk)
-        umma_bf16(dS, da + so + 2 * kk, dg + so + 2 * kk, X::IDESC_S,
-                  (k > par || kk > 0) ? 1u : 0u);
-      umma_commit(empty0 + 8 * st);
+        umma_bf16(tS, da + so + 2 * kk, dg + so + 2 * kk, X::IDESC_S, (k > 0 || kk > 0) ? 1u : 0u);
+      umma_commit(eb);
     }
-    if (good) umma_commit(s_full);  // (arrives at once when this half has no k-block)
-    if (par) {
-      if (!good) *abort_flag = 1;
-      goto xf_done;
-    }
+    if (good) umma_commit(s_full);
     // P V once every row's P is in TMEM and V has landed
     if (good && mbar_wait(p_ready, 0, abort_flag) && mbar_wait(v_full, 0, abort_flag)) {
       tc_fence_after();
@@ -1155,7 +1157,7 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     } else {
       *abort_flag = 1;
     }
-  } else if (live && warp >= 2 && warp < 6) {
+  } else if (warp >= 2 && warp < 6) {
     // ------------------------------------------------------------ softmax
     const int sp = warp & 3;
     const int row = sp * 32 + lane;
@@ -1172,18 +1174,6 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
       for (int i = 0; i < XK / 16; ++i) tmem_ld16_nowait(tS + lane_off + 16u * i, r + 16 * i);
       tmem_wait_ld();
-      if (nkb > 1) {  // S = S0 + S1 (the odd k-blocks)
-#pragma unroll
-        for (int j = 0; j < XK / 32; ++j) {
-          uint32_t q[32];
-          tmem_ld16_nowait(tS1 + lane_off + 32u * j, q);
-          tmem_ld16_nowait(tS1 + lane_off + 32u * j + 16u, q + 16);
-          tmem_wait_ld();
-#pragma unroll
-          for (int c = 0; c < 32; ++c)
-            r[32 * j + c] = __float_as_uint(__uint_as_float(r[32 * j + c]) + __uint_as_float(q[c]));
-        }
-      }
 #pragma unroll
       for (int c = 0; c < XK; ++c)
         r[c] = c < Nk ? __float_as_uint(__uint_as_float(r[c]) + s_kb[c])
@@ -1265,14 +1255,13 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       }
     }
   }
-xf_done:
-  if (live && (!ok || *abort_flag) && threadIdx.x == 64) atomicOr(err, DEVERR_TIMEOUT);
+  if ((!ok || *abort_flag) && threadIdx.x == 64) atomicOr(err, DEVERR_TIMEOUT);
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, 512);
+    tmem_dealloc(tmem_base, 256);
   }
 }
 
