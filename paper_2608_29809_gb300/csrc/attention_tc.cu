@@ -1009,11 +1009,17 @@ xattn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 // xb G_h^T + kb_h, G_h = K_h W_xq,h, kb_h = K_h b_h (a reassociation of the
 // same products).  The cross-query GEMM then disappears from the block.
 
-// One (query tile, head) per CTA: S = xb_tile G_h^T accumulated over d in
+// A unit is one (query tile, head): S = xb_tile G_h^T accumulated over d in
 // 64-column k-blocks (TMA ring, M = 128, N = 128), then the softmax of
-// (S + kb) / sqrt(dh) per row, P over S in TMEM, O = P V, O / l stored.
-// One warp loads the keys and V (from before the dependency wait on), one the
-// rows, one issues the MMAs with the next stage tested ahead.
+// (S + kb) / sqrt(dh) per row, P over S in TMEM, O = P V, O / l stored.  One
+// warp loads the keys and V (from before the dependency wait on), one the
+// rows, one issues the MMAs with the next stage tested ahead.  Persistent, at
+// most one CTA an SM: the units go round robin, S alternates between two
+// regions, and the P V of a unit is issued two thirds into the next unit's
+// S, so the softmax and the stores run under the MMAs.  (A CTA a unit of the
+// row bound, the ones past the live rows leaving at once, kept the next
+// kernel from starting until all had come and gone: 1024 px step 2640 us, 2594
+// now; eight 512 px sessions 3694 us, 3505 now.)
 constexpr int XF_STAGES = 6;
 constexpr int XF_THREADS = 224;  // rows, MMA, 4 softmax warps, keys and V
 template <int DH>
@@ -1023,8 +1029,7 @@ struct XFCfg {
   static constexpr int STAGE = STAGE_A + STAGE_G;
   static constexpr int V_ATOM = XK * 128;
   static constexpr int V_BYTES = C::TAIL ? 2 * V_ATOM : V_ATOM;
-  static constexpr size_t SMEM =
-      size_t(XF_STAGES) * STAGE + V_BYTES + XK * 4 + 1024 + 256;
+  static constexpr size_t SMEM = size_t(XF_STAGES) * STAGE + V_BYTES + 1024 + 256;
   static constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) |
                                       (uint32_t(XK >> 3) << 17) | (uint32_t(BQ >> 4) << 24);
 };
@@ -1042,13 +1047,12 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
   uint8_t* sV = smem + XF_STAGES * X::STAGE;
-  float* s_kb = reinterpret_cast<float*>(sV + X::V_BYTES);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(s_kb + XK);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sV + X::V_BYTES);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * XF_STAGES + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const uint32_t full0 = saddr(bars), empty0 = saddr(bars + XF_STAGES);
-  const uint32_t v_full = saddr(bars + 2 * XF_STAGES), s_full = v_full + 8, p_ready = v_full + 16,
-                 o_full = v_full + 24, kb_ready = v_full + 32;
+  const uint32_t v_full = saddr(bars + 2 * XF_STAGES), p_ready = v_full + 8, o_full = v_full + 16,
+                 s_full = v_full + 24;  // two, by S region
   const int warp = warp_index(), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int i = 0; i < XF_STAGES; ++i) {
@@ -1056,10 +1060,10 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       mbar_init(empty0 + 8 * i, 1);
     }
     mbar_init(v_full, 1);
-    mbar_init(s_full, 1);
     mbar_init(p_ready, 128);
     mbar_init(o_full, 1);
-    mbar_init(kb_ready, 128);
+    mbar_init(s_full, 1);
+    mbar_init(s_full + 8, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1069,20 +1073,17 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   // count and the turn's folded keys, key biases and text values.  Only the
   // bf16 rows of x come from the predecessor.
   const int D = live_count(rm.count, rm.bound, err);
-  const int qtiles = query_tiles(rm, xi.n, D);
-  const int qt = int(blockIdx.x) / heads, h = int(blockIdx.x) - (int(blockIdx.x) / heads) * heads;
-  // the grid covers the bound of the query tiles: CTAs past the live ones
-  // leave at once, before taking tensor memory
-  if (qt >= qtiles) return;
-  const TileLoc tl = locate_tile(rm, xi.n, D, qt);
-  if (warp == 1) tmem_alloc(saddr(tmem_slot), 256);
+  const int units = query_tiles(rm, xi.n, D) * heads;
+  // CTAs past the live units leave at once, before taking tensor memory
+  if (int(blockIdx.x) >= units) return;
+  if (warp == 1) tmem_alloc(saddr(tmem_slot), 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  // S | O; P is written over S
-  const uint32_t tS = tmem_base, tO = tmem_base + XK;
-  const int nkb = d / 64;
+  // S0 | S1 | O; P is written over its S
+  const uint32_t tO = tmem_base + 2 * XK;
+  const int nkb = d / 64, at_pv = 2 * nkb / 3;
   bool ok = true;
   if (warp == 0) {
     // ------------------------------------------------------------ TMA: rows
@@ -1091,93 +1092,131 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (elect_one()) {
       int st = 0;
       uint32_t ph = 1;
-      for (int k = 0; k < nkb; ++k) {
-        if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
-          *abort_flag = 1;
-          break;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+        const int row0 = locate_tile(rm, xi.n, D, u / heads).row0;
+        for (int k = 0; k < nkb; ++k) {
+          if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
+            ok = false;
+            break;
+          }
+          // (the keys may arrive before this expectation: the phase still
+          // needs this arrival)
+          mbar_expect_tx(full0 + 8 * st, X::STAGE);
+          tma_load_3d(saddr(smem + st * X::STAGE), &tmA, full0 + 8 * st, 0, k, row0);
+          if (++st == XF_STAGES) { st = 0; ph ^= 1; }
         }
-        // (the keys may arrive before this expectation: the phase still
-        // needs this arrival)
-        mbar_expect_tx(full0 + 8 * st, X::STAGE);
-        tma_load_3d(saddr(smem + st * X::STAGE), &tmA, full0 + 8 * st, 0, k, tl.row0);
-        if (++st == XF_STAGES) { st = 0; ph ^= 1; }
       }
+      if (!ok) *abort_flag = 1;
     }
   } else if (warp == 6) {
     // ------------------------------------------------------------ TMA: keys, V
     if (elect_one()) {
-      const int grow = xi.grow[tl.item] + h * XK;
       int st = 0;
       uint32_t ph = 1;
-      for (int k = 0; k < nkb; ++k) {
-        if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
-          *abort_flag = 1;
-          break;
-        }
-        tma_load_3d(saddr(smem + st * X::STAGE + X::STAGE_A), &tmG, full0 + 8 * st, 0, k, grow);
-        if (++st == XF_STAGES) { st = 0; ph ^= 1; }
-        if (k == (nkb < XF_STAGES ? nkb : XF_STAGES) - 1) {  // the ring is filled: V
-          mbar_expect_tx(v_full, X::V_BYTES);
-          tma_load_3d(saddr(sV), &tmV, v_full, 0, h, xi.vrow[tl.item]);
-          if (C::TAIL) tma_load_3d(saddr(sV + X::V_ATOM), &tmV, v_full, 64, h, xi.vrow[tl.item]);
+      int n = 0;  // units so far
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++n) {
+        const int qt = u / heads, h = u - qt * heads, item = locate_tile(rm, xi.n, D, qt).item;
+        const int grow = xi.grow[item] + h * XK;
+        // V once the ring is filled, or (the one buffer) at the end of a
+        // later unit, when the previous P V has read it
+        const int at_v = n ? nkb - 1 : (nkb < XF_STAGES ? nkb : XF_STAGES) - 1;
+        for (int k = 0; k < nkb; ++k) {
+          if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
+            ok = false;
+            break;
+          }
+          tma_load_3d(saddr(smem + st * X::STAGE + X::STAGE_A), &tmG, full0 + 8 * st, 0, k, grow);
+          if (++st == XF_STAGES) { st = 0; ph ^= 1; }
+          if (k == at_v) {
+            if (n && !mbar_wait(o_full, (n - 1) & 1, abort_flag)) {
+              ok = false;
+              break;
+            }
+            mbar_expect_tx(v_full, X::V_BYTES);
+            tma_load_3d(saddr(sV), &tmV, v_full, 0, h, xi.vrow[item]);
+            if (C::TAIL) tma_load_3d(saddr(sV + X::V_ATOM), &tmV, v_full, 64, h, xi.vrow[item]);
+          }
         }
       }
+      if (!ok) *abort_flag = 1;
     }
-  } else if (warp == 1 && elect_one()) {
+  } else if (warp == 1) {
     // ------------------------------------------------------------ MMA
-    const uint64_t da = sw128_desc(saddr(smem)), dg = sw128_desc(saddr(smem + X::STAGE_A));
-    bool good = true, ready = false;
-    int st = 0;
-    uint32_t ph = 0;
-    for (int k = 0; k < nkb; ++k) {
-      if (!ready && !mbar_wait(full0 + 8 * st, ph, abort_flag)) {
-        good = false;
-        break;
-      }
-      const uint64_t so = uint64_t((st * X::STAGE) >> 4);
-      const uint32_t eb = empty0 + 8 * st;
-      if (++st == XF_STAGES) { st = 0; ph ^= 1; }
-      ready = mbar_test(full0 + 8 * st, ph);  // (beside this stage's MMAs)
-      tc_fence_after();
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
-        umma_bf16(tS, da + so + 2 * kk, dg + so + 2 * kk, X::IDESC_S, (k > 0 || kk > 0) ? 1u : 0u);
-      umma_commit(eb);
-    }
-    if (good) umma_commit(s_full);
-    // P V once every row's P is in TMEM and V has landed
-    if (good && mbar_wait(p_ready, 0, abort_flag) && mbar_wait(v_full, 0, abort_flag)) {
-      tc_fence_after();
+    if (elect_one()) {
+      const uint64_t da = sw128_desc(saddr(smem)), dg = sw128_desc(saddr(smem + X::STAGE_A));
       const uint64_t dv = C::TAIL ? sw128_mnmajor_desc_lbo(saddr(sV), X::V_ATOM)
                                   : sw128_mnmajor_desc(saddr(sV));
+      // P V of the n-th unit once every row's P is in TMEM (and the previous
+      // O read) and V has landed
+      auto pv = [&](int n) -> bool {
+        if (!mbar_wait(p_ready, n & 1, abort_flag) || !mbar_wait(v_full, n & 1, abort_flag))
+          return false;
+        tc_fence_after();
+        const uint32_t tP = tmem_base + uint32_t(n & 1) * XK;
 #pragma unroll
-      for (int kk = 0; kk < XK / 16; ++kk)
-        umma_bf16_ta(tO, tS + 8 * kk, dv + 128 * kk, C::IDESC_PV, kk > 0 ? 1u : 0u);
-      umma_commit(o_full);
-    } else {
-      *abort_flag = 1;
+        for (int kk = 0; kk < XK / 16; ++kk)
+          umma_bf16_ta(tO, tP + 8 * kk, dv + 128 * kk, C::IDESC_PV, kk > 0 ? 1u : 0u);
+        umma_commit(o_full);
+        return true;
+      };
+      bool ready = false;
+      int st = 0, n = 0;
+      uint32_t ph = 0;
+      for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++n) {
+        // the S region: its last reader was the P V of two units ago
+        if (n >= 2 && !mbar_wait(o_full, n & 1, abort_flag)) ok = false;
+        const uint32_t tS = tmem_base + uint32_t(n & 1) * XK;
+        for (int k = 0; k < nkb && ok; ++k) {
+          if (!ready && !mbar_wait(full0 + 8 * st, ph, abort_flag)) {
+            ok = false;
+            break;
+          }
+          const uint64_t so = uint64_t((st * X::STAGE) >> 4);
+          const uint32_t eb = empty0 + 8 * st;
+          if (++st == XF_STAGES) { st = 0; ph ^= 1; }
+          ready = mbar_test(full0 + 8 * st, ph);  // (beside this stage's MMAs)
+          tc_fence_after();
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            umma_bf16(tS, da + so + 2 * kk, dg + so + 2 * kk, X::IDESC_S,
+                      (k > 0 || kk > 0) ? 1u : 0u);
+          umma_commit(eb);
+          if (n && k == at_pv) ok = pv(n - 1);
+        }
+        if (ok) umma_commit(s_full + 8 * (n & 1));
+      }
+      if (!(ok && pv(n - 1))) *abort_flag = 1;
     }
-  } else if (warp >= 2 && warp < 6) {
+  } else {
     // ------------------------------------------------------------ softmax
     const int sp = warp & 3;
     const int row = sp * 32 + lane;
     const uint32_t lane_off = uint32_t(sp * 32) << 16;
-    const int t128 = threadIdx.x - 64;  // 0 .. 127
-    s_kb[t128] = t128 < Nk ? kb[size_t(xi.grow[tl.item]) + size_t(h) * XK + t128] : 0.f;
     pdl_wait();  // (before any global write: the predecessor reads O's buffer)
-    mbar_arrive(kb_ready);
-    ok = mbar_sleep_warp(kb_ready, 0, abort_flag) && mbar_sleep_warp(s_full, 0, abort_flag);
-    float l = 0.f;
-    if (ok) {
+    int n = 0;
+    for (int u = blockIdx.x; u < units && ok; u += gridDim.x, ++n) {
+      const int qt = u / heads, h = u - qt * heads;
+      const TileLoc tl = locate_tile(rm, xi.n, D, qt);
+      const float4* b4 =
+          reinterpret_cast<const float4*>(kb + size_t(xi.grow[tl.item]) + size_t(h) * XK);
+      const uint32_t tS = tmem_base + uint32_t(n & 1) * XK + lane_off;
+      ok = mbar_sleep_warp(s_full + 8 * (n & 1), (n >> 1) & 1, abort_flag);
+      if (!ok) break;
       tc_fence_after();
       uint32_t r[XK];
 #pragma unroll
-      for (int i = 0; i < XK / 16; ++i) tmem_ld16_nowait(tS + lane_off + 16u * i, r + 16 * i);
+      for (int i = 0; i < XK / 16; ++i) tmem_ld16_nowait(tS + 16u * i, r + 16 * i);
       tmem_wait_ld();
 #pragma unroll
-      for (int c = 0; c < XK; ++c)
-        r[c] = c < Nk ? __float_as_uint(__uint_as_float(r[c]) + s_kb[c])
-                      : __float_as_uint(-INFINITY);
+      for (int c = 0; c < XK / 4; ++c) {
+        const float4 t = __ldg(b4 + c);
+        const float a[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          r[4 * c + e] = 4 * c + e < Nk
+                             ? __float_as_uint(__uint_as_float(r[4 * c + e]) + a[e])
+                             : __float_as_uint(-INFINITY);
+      }
       float mx8[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) mx8[q] = __uint_as_float(r[q]);
@@ -1205,7 +1244,7 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       unpack_f32x2(sum2[1], s2, s3);
       unpack_f32x2(sum2[2], s4, s5);
       unpack_f32x2(sum2[3], s6, s7);
-      l = ((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7));
+      const float l = ((s0 + s1) + (s2 + s3)) + ((s4 + s5) + (s6 + s7));
       if (CAP && cap.n && row < tl.rows) {  // the localisation scores of the listed keys
         const int qrow = tl.row0 + row;
         const int tok = rm.tok ? __ldg(rm.tok + qrow) : qrow;
@@ -1227,14 +1266,13 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         for (int c = 0; c < 16; ++c)
           w[c] = pack_bf16x2(__uint_as_float(r[32 * h2 + 2 * c]),
                              __uint_as_float(r[32 * h2 + 2 * c + 1]));
-        tmem_st16(tS + lane_off + 16u * h2, w);
+        tmem_st16(tS + 16u * h2, w);
       }
       tmem_wait_st();
-    }
-    tc_fence_before();
-    mbar_arrive(p_ready);  // arrives even on failure so that no wait is left open
-    if (ok) ok = mbar_sleep_warp(o_full, 0, abort_flag);
-    if (ok) {
+      tc_fence_before();
+      mbar_arrive(p_ready);
+      ok = mbar_sleep_warp(o_full, n & 1, abort_flag);
+      if (!ok) break;
       tc_fence_after();
       uint32_t o[C::DHP];
 #pragma unroll
@@ -1254,6 +1292,7 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
       }
     }
+    if (!ok) *abort_flag = 1;
   }
   if ((!ok || *abort_flag) && threadIdx.x == 64) atomicOr(err, DEVERR_TIMEOUT);
   tc_fence_before();
@@ -1261,7 +1300,7 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, 256);
+    tmem_dealloc(tmem_base, 512);
   }
 }
 
@@ -1469,7 +1508,8 @@ cudaError_t launch_xattn_fused(const bf16* xb, int ldx, const bf16* G, const flo
     if (xi.grow[i] < 0 || xi.grow[i] + heads * XK > g_rows || xi.vrow[i] < 0 ||
         xi.vrow[i] > v_rows - Nk)
       return cudaErrorInvalidValue;
-  if (!device_sms_attn()) return cudaErrorInvalidDevice;
+  const int sms = device_sms_attn();
+  if (!sms) return cudaErrorInvalidDevice;
   AttnCapture cap{};
   if (capture && capture->n > 0) {
     if (capture->n > 8 || !capture->out) return cudaErrorInvalidValue;
@@ -1488,8 +1528,8 @@ cudaError_t launch_xattn_fused(const bf16* xb, int ldx, const bf16* G, const flo
   if (grid >= (1ll << 31)) return cudaErrorInvalidValue;
   auto fn = dh == 72 ? (cap.n ? xfused_tc_kernel<72, true> : xfused_tc_kernel<72, false>)
                      : (cap.n ? xfused_tc_kernel<64, true> : xfused_tc_kernel<64, false>);
-  RC_TRY(launch_k(fn, dim3(unsigned(grid)), dim3(XF_THREADS), dh == 72 ? XFCfg<72>::SMEM : XFCfg<64>::SMEM,
-                  st, ta, tg, tv, kb, xi, Nk, d, O, ldo, heads, rm, scale_log2, err, cap));
+  RC_TRY(launch_k(fn, dim3(unsigned(grid < sms ? grid : sms)), dim3(XF_THREADS),
+                  dh == 72 ? XFCfg<72>::SMEM : XFCfg<64>::SMEM, st, ta, tg, tv, kb, xi, Nk, d, O, ldo, heads, rm, scale_log2, err, cap));
   count_launches(1);
   return cudaSuccess;
 }

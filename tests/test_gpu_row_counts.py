@@ -1,5 +1,6 @@
 """One block at row counts around the 128-row tiles of its GEMMs, where the
-split of a matrix's k range changes (up to eight parts for one row tile),
+split of a matrix's k range changes (up to eight parts for one row tile) and
+where the folded cross-attention's CTAs take one or two (tile, head) units,
 against the oracle."""
 import dataclasses
 
@@ -19,12 +20,12 @@ def problem():
     from paper_2608_29809_gb300 import build as B
     B.build()
     from paper_2608_29809_gb300 import regioncache as R
-    p = Problem(R, dataclasses.replace(synth.ONE_BLOCK_256, grid_h=32, grid_w=32), 4321)
+    p = Problem(R, dataclasses.replace(synth.ONE_BLOCK_256, grid_h=48, grid_w=48), 4321)
     yield p
     p.close()
 
 
-@pytest.mark.parametrize("rows", [1, 128, 129, 256, 385, 640, 897])
+@pytest.mark.parametrize("rows", [1, 128, 129, 256, 385, 640, 897, 1217, 2047])
 def test_block_at_row_tile_edges(problem, rows):
     p, d = problem, problem.d
     idx = np.sort(np.random.default_rng(rows).choice(d.tokens, rows, replace=False))
