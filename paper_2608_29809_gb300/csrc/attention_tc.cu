@@ -398,8 +398,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   AttnUnits un;
   un.init(pt, rm, ai.n, D, heads, Nk, int(gridDim.x));
   const int u0 = blockIdx.x, du = gridDim.x;
-  pdl_wait();
-  pdl_trigger();
+  // the roles wait for the predecessor where they first need it: what comes
+  // before (the first unit's place, and fetching the code that finds it) runs
+  // beside the predecessor's end
 
   if (warp == 0) {
     // ------------------------------------------------------------ Q and K
@@ -411,6 +412,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       const TileLoc tl = locate_group(rm, ai.n, D, un.rows, w.g);
       const int krow = ai.krow[tl.item], tiles = tl.rows > BQ ? 2 : 1;
       if (!mbar_sleep_warp(q_empty, (uc & 1) ^ 1, abort_flag)) goto timeout;
+      if (uc == 0) {
+        pdl_wait();
+        pdl_trigger();
+      }
       if (leader) {
         mbar_expect_tx(q_full, tiles * C::Q_BYTES);
         for (int x = 0; x < tiles; ++x) {
@@ -435,6 +440,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       // (the next unit's Q waits for this one's last S, which waits for these)
       if (C::TAIL) tell_tails<0>(g, told, k_full, KS, lane);
     }
+    if (uc == 0) pdl_wait();  // (no kernel ends before its predecessor has)
   } else if (warp == 1 || warp == 3) {
     // ------------------------------------------- S = Q K^T and O += P V of a stream
     // S runs up to two of the stream's blocks ahead (two buffers); a buffer
@@ -512,6 +518,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     for (int u = u0; u < un.units; u += du) {
       w.set(un, u);
       const int vrow = ai.vrow[locate_group(rm, ai.n, D, un.rows, w.g).item];
+      if (g == 0) pdl_wait();
       for (int kb = w.kb0; kb < w.kb1; ++kb, ++g) {
         const int s = g % VS;
         if (!mbar_sleep_warp(v_empty + 8 * s, ((g / VS) & 1) ^ 1, abort_flag)) goto timeout;
@@ -551,6 +558,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       const int n = w.kb1 - w.kb0;
       const TileLoc tl = locate_group(rm, ai.n, D, un.rows, w.g);
       const bool two = tl.rows > BQ;
+      if (uc == 0) pdl_wait();  // (before any global write)
       float m = -INFINITY, l = 0.f;
       float cap_s[8];  // scaled scores of the captured key columns
 #pragma unroll
@@ -1074,8 +1082,12 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   // bf16 rows of x come from the predecessor.
   const int D = live_count(rm.count, rm.bound, err);
   const int units = query_tiles(rm, xi.n, D) * heads;
-  // CTAs past the live units leave at once, before taking tensor memory
-  if (int(blockIdx.x) >= units) return;
+  // CTAs past the live units leave before taking tensor memory (but no kernel
+  // ends before its predecessor has)
+  if (int(blockIdx.x) >= units) {
+    pdl_wait();
+    return;
+  }
   if (warp == 1) tmem_alloc(saddr(tmem_slot), 512);
   tc_fence_before();
   __syncthreads();
@@ -1087,13 +1099,15 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   bool ok = true;
   if (warp == 0) {
     // ------------------------------------------------------------ TMA: rows
-    pdl_wait();
-    pdl_trigger();
     if (elect_one()) {
       int st = 0;
       uint32_t ph = 1;
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
         const int row0 = locate_tile(rm, xi.n, D, u / heads).row0;
+        if (u == int(blockIdx.x)) {
+          pdl_wait();
+          pdl_trigger();
+        }
         for (int k = 0; k < nkb; ++k) {
           if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
             ok = false;
@@ -1200,6 +1214,9 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const float4* b4 =
           reinterpret_cast<const float4*>(kb + size_t(xi.grow[tl.item]) + size_t(h) * XK);
       const uint32_t tS = tmem_base + uint32_t(n & 1) * XK + lane_off;
+      // (the key biases are fetched into L1 beside the product)
+      const float4 warm = __ldg(b4 + lane);
+      asm volatile("" ::"f"(warm.x));
       ok = mbar_sleep_warp(s_full + 8 * (n & 1), (n >> 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();

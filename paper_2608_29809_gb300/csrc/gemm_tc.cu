@@ -493,8 +493,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
   if (warp == 0) {
     // ------------------------------------------------------- TMA producer
-    pdl_wait();
-    pdl_trigger();
     if (elect_one()) {
       // W as one box of BN rows, or BN / 2 rows per CTA of a pair (maps for
       // the heights that divide n)
@@ -505,9 +503,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       Segs sg;
       sg.init(sc, pos);
       int t, kb0, kb1;
+      bool waited = false;
       while (sg.next(t, kb0, kb1)) {
         const int mq = t % sc.mt, nn = t / sc.mt;
         const int m = PAIR ? 2 * mq + int(rank) : mq;
+        if (!waited) {  // (the first tile's place was found beside the predecessor's end)
+          waited = true;
+          pdl_wait();
+          pdl_trigger();
+        }
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag)) goto timeout;
           uint8_t* st = smem + stage * STAGE;
@@ -527,6 +531,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
       }
+      if (!waited) pdl_wait();  // (no kernel ends before its predecessor has)
     }
   } else if (warp == W_WARP) {
     // ------------------------------------------------------- TMA: W (unpaired)
