@@ -156,7 +156,9 @@ def _ptr(t):
 
 def _stream(stream):
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # the current stream's handle without a Stream object around it (3.0 us
+        # a call with one, 0.3 without)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
 
 
