@@ -412,12 +412,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       const TileLoc tl = locate_group(rm, ai.n, D, un.rows, w.g);
       const int krow = ai.krow[tl.item], tiles = tl.rows > BQ ? 2 : 1;
       if (!mbar_sleep_warp(q_empty, (uc & 1) ^ 1, abort_flag)) goto timeout;
+      if (leader) mbar_expect_tx(q_full, tiles * C::Q_BYTES);
       if (uc == 0) {
         pdl_wait();
         pdl_trigger();
       }
       if (leader) {
-        mbar_expect_tx(q_full, tiles * C::Q_BYTES);
         for (int x = 0; x < tiles; ++x) {
           uint8_t* q = sQ + x * C::Q_BYTES;
           tma_load_3d(saddr(q), &tmQ, q_full, 0, w.h, tl.row0 + x * BQ);
@@ -518,10 +518,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     for (int u = u0; u < un.units; u += du) {
       w.set(un, u);
       const int vrow = ai.vrow[locate_group(rm, ai.n, D, un.rows, w.g).item];
-      if (g == 0) pdl_wait();
       for (int kb = w.kb0; kb < w.kb1; ++kb, ++g) {
         const int s = g % VS;
         if (!mbar_sleep_warp(v_empty + 8 * s, ((g / VS) & 1) ^ 1, abort_flag)) goto timeout;
+        if (g == 0) pdl_wait();
         if (leader) {
           mbar_expect_tx(v_full + 8 * s, C::K128);
           tma_load_3d(saddr(sV + C::v_main(s)), &tmV, v_full + 8 * s, 0, w.h, vrow + kb * BKV);
@@ -1102,12 +1102,9 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (elect_one()) {
       int st = 0;
       uint32_t ph = 1;
+      bool waited = false;
       for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
         const int row0 = locate_tile(rm, xi.n, D, u / heads).row0;
-        if (u == int(blockIdx.x)) {
-          pdl_wait();
-          pdl_trigger();
-        }
         for (int k = 0; k < nkb; ++k) {
           if (!mbar_wait(empty0 + 8 * st, ph, abort_flag)) {
             ok = false;
@@ -1116,6 +1113,11 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
           // (the keys may arrive before this expectation: the phase still
           // needs this arrival)
           mbar_expect_tx(full0 + 8 * st, X::STAGE);
+          if (!waited) {  // (everything up to the first load runs beside the predecessor's end)
+            waited = true;
+            pdl_wait();
+            pdl_trigger();
+          }
           tma_load_3d(saddr(smem + st * X::STAGE), &tmA, full0 + 8 * st, 0, k, row0);
           if (++st == XF_STAGES) { st = 0; ph ^= 1; }
         }

@@ -507,25 +507,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       while (sg.next(t, kb0, kb1)) {
         const int mq = t % sc.mt, nn = t / sc.mt;
         const int m = PAIR ? 2 * mq + int(rank) : mq;
-        if (!waited) {  // (the first tile's place was found beside the predecessor's end)
-          waited = true;
-          pdl_wait();
-          pdl_trigger();
-        }
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag)) goto timeout;
           uint8_t* st = smem + stage * STAGE;
+          // (for a pair both CTAs' bytes land on rank 0's barrier)
+          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, PAIR ? 2 * STAGE : STAGE);
+          if (!waited) {  // (everything up to the first load runs beside the predecessor's end)
+            waited = true;
+            pdl_wait();
+            pdl_trigger();
+          }
           if (PAIR) {
-            // both CTAs' bytes land on rank 0's barrier, which expects them
             const uint32_t fb = mapa_shared(full0 + 8 * stage, 0);
-            if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * STAGE);
             tma_load_2d_pair(saddr(st), &tmA, fb, kb * BK, m * BM);
             tma_load_2d_pair(saddr(st + STAGE_A), tmW, fb, kb * BK, nn * BN + int(rank) * brows);
           } else {
             // W comes from the W warp on the same barrier (which may see
             // its bytes before this expectation: the phase still needs this
             // arrival)
-            mbar_expect_tx(full0 + 8 * stage, STAGE);
             tma_load_2d(saddr(st), &tmA, full0 + 8 * stage, kb * BK, m * BM);
           }
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
