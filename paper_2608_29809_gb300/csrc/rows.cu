@@ -373,7 +373,11 @@ cudaError_t launch_localize(const float* A, int S, int N, int M, int gh, int gw,
 // once, and consecutive rows go to different CTAs, so that few rows spread
 // over the whole chip.  (Four warps per row halve a row's chain but double its
 // instructions: 4096 rows took 13.5 us that way, 8.3 this way; 831 rows 4.9
-// and 3.7.)
+// and 3.7.)  With several items a CTA takes neighbouring rows instead, nearly
+// always one item's, and stages that item's vectors; a row of another item
+// fetches its own.  (Every row doing so took 6.0 us after the dependency wait
+// for 1500 rows of eight items; eight 512 px sessions 3485 us a step, 3406 now.
+// One item's kernel, without the choice: 1024 px step 2584 -> 2564 us.)
 constexpr int LN_WARPS = 8, LN_CTAS = 3;
 constexpr int LN_MAXV = 12;  // float4 per lane
 constexpr int LN_SV = (LN_MAXV * 32 + LN_WARPS * 32 - 1) / (LN_WARPS * 32);  // float4 per thread
@@ -398,13 +402,13 @@ __device__ __forceinline__ bool row_target(const RowMap& rm, int n_items, int r,
   return row_valid(rm, n_items, tok, item, err, lane);
 }
 
+template <bool MANY>
 __global__ void __launch_bounds__(LN_WARPS * 32, LN_CTAS)
 ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
               const float* __restrict__ tab, int k_sh, int k_sc,
               const __grid_constant__ Items it, bf16* __restrict__ out, RowMap rm,
               long long hprev_off, int d, unsigned* err) {
-  // shift and scale staged once per CTA: tab (+ the item's tb when the
-  // launch has one item; otherwise each row adds its item's tb).
+  // shift and scale staged once per CTA: tab + the tb of its (first row's) item.
   // The vectors and the row count are requested before the programmatic-
   // dependency wait: every kernel here waits for its predecessor before
   // letting its successor start, so whatever was written two or more launches
@@ -416,7 +420,19 @@ ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
   const int lane = threadIdx.x & 31;
   const int nv = d / 128, nq = d / 4;
   if (x_copy) pdl_wait();
-  const float* tb0 = it.n == 1 ? it.tb[0] : nullptr;
+  // rows r0 + step * warp .. below D: dealt round robin, or (several items)
+  // this CTA's neighbouring rows
+  int r0 = blockIdx.x, D = 0, staged = 0;
+  const int step = MANY ? 1 : gridDim.x;
+  if (MANY) {
+    D = live_count(rm.count, rm.bound, err);
+    const int share = (D + int(gridDim.x) - 1) / int(gridDim.x);
+    r0 = int(blockIdx.x) * share;
+    D = min(D, r0 + share);
+    staged = r0 < D && rm.item ? __ldg(rm.item + r0) : 0;
+    if (staged < 0 || staged >= it.n) staged = 0;
+  }
+  const float* tb0 = it.tb[staged];
   float4 m[4][LN_SV];  // tab shift, tab scale, tb shift, tb scale
 #pragma unroll
   for (int j = 0; j < LN_SV; ++j) {
@@ -432,7 +448,7 @@ ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
       m[3][j] = __ldg(reinterpret_cast<const float4*>(tb0 + size_t(k_sc) * d) + q);
     }
   }
-  const int D = live_count(rm.count, rm.bound, err);
+  if (!MANY) D = live_count(rm.count, rm.bound, err);
 #pragma unroll
   for (int j = 0; j < LN_SV; ++j) {
     const int q = threadIdx.x + j * LN_WARPS * 32;
@@ -449,7 +465,7 @@ ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
   __syncthreads();
   pdl_wait();
   pdl_trigger();
-  for (int r = blockIdx.x + gridDim.x * (threadIdx.x >> 5); r < D; r += gridDim.x * LN_WARPS) {
+  for (int r = r0 + step * (threadIdx.x >> 5); r < D; r += step * LN_WARPS) {
     const int tok = rm.tok ? __ldg(rm.tok + r) : r;
     const int item = rm.item ? __ldg(rm.item + r) : 0;
     if (x_copy && !row_valid(rm, it.n, tok, item, err, lane)) continue;
@@ -486,7 +502,7 @@ ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
         q += (v[k].x * v[k].x + v[k].y * v[k].y) + (v[k].z * v[k].z + v[k].w * v[k].w);
       }
     const float rstd = 1.0f / sqrtf(warp_sum(q) / float(d) + 1e-6f);
-    const float* tb = tb0 ? nullptr : it.tb[item];
+    const float* tb = !MANY || item == staged ? nullptr : it.tb[item];
     uint2* orow = reinterpret_cast<uint2*>(out + size_t(r) * d);
 #pragma unroll
     for (int k = 0; k < LN_MAXV; ++k)
@@ -494,7 +510,10 @@ ln_mod_kernel(const float* __restrict__ x, float* __restrict__ x_copy,
         const int c = 4 * (lane + 32 * k);
         float4 sh = *reinterpret_cast<const float4*>(s_mod + c);
         float4 sc = *reinterpret_cast<const float4*>(s_mod + d + c);
-        if (tb) {
+        if (MANY && tb) {
+          const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+          sh = tab ? __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sh) * d + c)) : zero;
+          sc = tab ? __ldg(reinterpret_cast<const float4*>(tab + size_t(k_sc) * d + c)) : zero;
           const float4 a = __ldg(reinterpret_cast<const float4*>(tb + size_t(k_sh) * d + c));
           const float4 b = __ldg(reinterpret_cast<const float4*>(tb + size_t(k_sc) * d + c));
           sh.x += a.x; sh.y += a.y; sh.z += a.z; sh.w += a.w;
@@ -512,8 +531,8 @@ cudaError_t launch_ln_mod(const float* x, float* x_copy, const float* tab, int k
                           unsigned* err, cudaStream_t st) {
   if (rm.bound <= 0) return cudaSuccess;
   if (d % 128 || d > 128 * LN_MAXV) return cudaErrorInvalidValue;
-  RC_TRY(launch_k(ln_mod_kernel, dim3(row_grid(rm.bound, 1, LN_CTAS)), dim3(LN_WARPS * 32),
-                  size_t(2) * d * sizeof(float), st, x, x_copy, tab, k_sh, k_sc, it, out, rm,
+  RC_TRY(launch_k(it.n > 1 ? ln_mod_kernel<true> : ln_mod_kernel<false>,
+                  dim3(row_grid(rm.bound, 1, LN_CTAS)), dim3(LN_WARPS * 32), size_t(2) * d * sizeof(float), st, x, x_copy, tab, k_sh, k_sc, it, out, rm,
                   hprev_off, d, err));
   count_launches(1);
   return cudaSuccess;

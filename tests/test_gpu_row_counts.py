@@ -10,7 +10,8 @@ import torch
 
 import oracle as O
 from paper_2608_29809_gb300 import synth
-from tests.gpu_cases import Problem, block_close
+from tests.gpu_cases import LATENT_REL_L2, Problem, block_close, rel_l2
+from tests.test_gpu_batched import Sessions
 
 pytestmark = pytest.mark.gpu
 
@@ -44,3 +45,33 @@ def test_block_at_row_tile_edges(problem, rows):
     after = p.read_slot(0, 0)
     for k in "HKV":
         block_close(after[k][idx], cache[k][idx], f"cache {k}")
+
+
+def test_batch_rows_of_neighbouring_items():
+    """Items whose rows meet within one CTA's share of the LayerNorm rows."""
+    from paper_2608_29809_gb300 import build as B
+    B.build()
+    from paper_2608_29809_gb300 import regioncache as R
+    d = dataclasses.replace(synth.PIXART_512, layers=1, timesteps=2)
+    S = Sessions(R, d, 4322, 3, max_batch=3)
+    try:
+        items, idxs, lats = [], [], []
+        for s, rows in enumerate((1, 457, 333)):
+            S.fill(s, s % 2)
+            idx = np.sort(np.random.default_rng(s).choice(d.tokens, rows, replace=False))
+            lat = synth.make_latent(d, 4322 + s)
+            items.append(dict(session=s, latent=lat.clone().cuda(), t=s % 2, mode=O.MODE_SPARSE,
+                              dirty_idx=torch.from_numpy(idx.astype(np.int32)).cuda(), D=rows,
+                              dirty_count=None))
+            idxs.append(idx)
+            lats.append(lat)
+        R.rc_step_batched(S.model.ctx, S.model.cache, items)
+        R.rc_sync(S.model.ctx)
+        for s, it in enumerate(items):
+            want, _, cache = S.oracle(s, O.to64(lats[s]), s % 2, O.MODE_SPARSE, idxs[s])
+            assert rel_l2(it["latent"].cpu().double().numpy(), want) <= LATENT_REL_L2, s
+            sl = S.read(s, 0, s % 2)
+            for k in "HKV":
+                block_close(sl[k][idxs[s]], cache[0][k][idxs[s]], f"session {s} {k}")
+    finally:
+        S.close()
