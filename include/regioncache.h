@@ -405,7 +405,7 @@ rc_status rc_prompt_similarity(const float* e_minus, const float* e_plus, int di
 rc_status rc_reuse_schedule(float s, float tau_s, float rho, int T, uint8_t* modes_out);
 
 /* CUDA Graph of one rc_step (no counterpart in the paper; serving
- * plumbing): the step's ~290 kernel launches for fixed arguments are
+ * plumbing): the step's ~255 kernel launches for fixed arguments are
  * recorded once and replayed with one launch call.  The arguments are those
  * of rc_step; the graph keeps the device pointers (latent, dirty_idx,
  * dirty_count, the cache slots of (session, t)) and reads and writes their

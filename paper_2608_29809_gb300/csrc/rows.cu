@@ -40,8 +40,9 @@ static inline int row_grid(int rows_bound, int rows_per_cta, int per_sm) {
 // the counts through its shared memory, so that the steps that need every
 // token's result of the previous one are cluster barriers instead of
 // launches.  1024 tokens, 5 delta tokens: 7.9 -> 5.9 us on the device (four
-// launches before), 17.9 -> 12.6 us a call from Python; 16384 tokens, 8 delta
-// tokens, 16 slices: 50 -> 32 us.
+// launches before), 17.9 -> 12.6 us a call from Python (8.3 since the binding
+// asks for the raw stream handle); 16384 tokens, 8 delta tokens, 16 slices:
+// 50 -> 32 us.
 // Workspace: abar f32 [n_delta][N] | part f32x2 [nblk][n_delta] | union u8 [N]
 // | cnt int [nblk] (the last two are unused and kept for the stated size).
 constexpr int MASK_ROWS = 256;
@@ -532,7 +533,8 @@ cudaError_t launch_ln_mod(const float* x, float* x_copy, const float* tab, int k
   if (rm.bound <= 0) return cudaSuccess;
   if (d % 128 || d > 128 * LN_MAXV) return cudaErrorInvalidValue;
   RC_TRY(launch_k(it.n > 1 ? ln_mod_kernel<true> : ln_mod_kernel<false>,
-                  dim3(row_grid(rm.bound, 1, LN_CTAS)), dim3(LN_WARPS * 32), size_t(2) * d * sizeof(float), st, x, x_copy, tab, k_sh, k_sc, it, out, rm,
+                  dim3(row_grid(rm.bound, 1, LN_CTAS)), dim3(LN_WARPS * 32),
+                  size_t(2) * d * sizeof(float), st, x, x_copy, tab, k_sh, k_sc, it, out, rm,
                   hprev_off, d, err));
   count_launches(1);
   return cudaSuccess;
