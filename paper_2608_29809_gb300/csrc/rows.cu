@@ -248,16 +248,19 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
     const float rng = __fsub_rn(hi, lo);
     s_mn[j] = lo;
     s_rng[j] = rng;
-    s_inv[j] = __fdiv_rn(1.f, rng);
+    // (NaN where the reciprocal overflows, for ranges below 2^-128: no product
+    // settles a comparison there)
+    const float inv = __fdiv_rn(1.f, rng);
+    s_inv[j] = isfinite(inv) ? inv : NAN;
     s_ok[j] = rng > 0.0f && lo != -INFINITY && hi != INFINITY;
   }
   __syncthreads();
   // the thresholded union to every CTA; a warp owns up to four words of 32
   // tokens, whose scores of several delta tokens are in flight together.  The
   // division is correctly rounded by definition and takes some 40
-  // instructions; the product with the reciprocal is within a few ulp of it,
-  // so it is taken only where that does not settle the comparison (NaN and
-  // overflowing products among them)
+  // instructions; the product with the reciprocal is within 4e-7 of it
+  // (relative), so the division is taken only where that does not settle the
+  // comparison, and wherever the product is NaN
   {
     bool u[MASK_WPW] = {};
     const float margin = fmaxf(1e-6f * fabsf(tau), 1e-37f);
