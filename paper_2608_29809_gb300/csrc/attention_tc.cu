@@ -133,8 +133,14 @@ struct ACfg {
   // K-major operands); V: one SW128 atom per 64 head-dim columns, so that P V
   // is a single MMA of N = DHP per 16 keys (MN-major B spanning the atoms).
   // Of the second atom only 32 bytes a row are used, so four stages share one
+  // A unit of one tile gives its blocks to the streams in turn, and a stream
+  // waits only for its own: with rings of even depth a stage then keeps its
+  // stream within a unit, so that a parity wait never meets a fill two ahead
+  // of the last one it saw.  (From one unit to the next q_full and o_free
+  // follow every K and V of the unit before.)
   static constexpr int K_STAGES = 6;
-  static constexpr int V_STAGES = 7;
+  static constexpr int V_STAGES = 8;
+  static_assert(K_STAGES % 2 == 0 && V_STAGES % 2 == 0, "a stage belongs to one stream of a unit");
   static constexpr int Q_BYTES = Q128 + Q32;
   static constexpr int K_STRIDE = (K128 + K32 + 1023) & ~1023;  // bytes between K stages
   static constexpr int V_TAILS = TAIL ? (V_STAGES + 3) / 4 : 0;
