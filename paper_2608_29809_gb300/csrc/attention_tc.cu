@@ -511,7 +511,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           umma_commit(v_empty + 8 * s);
           if (!two) umma_commit(v_empty + 8 * s);
         }
-        if (i0 >= n) umma_commit(q_empty);  // (no block in this unit)
+        if (i0 >= n) {
+          // no block in this unit: o_full counts each stream once a unit, so
+          // this one is told only when the unit before has been read
+          umma_commit(q_empty);
+          if (!mbar_sleep(o_free, (uc & 1) ^ 1, abort_flag)) goto timeout;
+        }
         umma_commit(o_full);
         g0 += n;
       }

@@ -1,7 +1,8 @@
 """The order that the self-attention kernel's barriers give, on a model of its
 warps (loads, the two issuing streams, the two softmax streams): every product
 reads the blocks that it is meant to read, however long each load takes.  The
-ring depths are the kernel's own, read from its source."""
+ring depths, and what a stream without a block waits for, are the kernel's own,
+read from its source."""
 import heapq
 import os
 import random
@@ -11,6 +12,8 @@ import pytest
 
 SRC = open(os.path.join(os.path.dirname(os.path.abspath(__file__)), os.pardir,
                         "paper_2608_29809_gb300", "csrc", "attention_tc.cu")).read()
+# a stream without a block in a unit waits for the O of the unit before
+EMPTY_WAITS = bool(re.search(r"if \(i0 >= n\) \{[^}]*mbar_sleep\(o_free", SRC))
 KS, VS = (int(re.search(rf"{n}_STAGES = (\d+);", SRC).group(1)) for n in "KV")
 
 
@@ -32,7 +35,7 @@ class Fault(Exception):
     pass
 
 
-def simulate(units, ks, vs, seed):
+def simulate(units, ks, vs, seed, empty_waits=EMPTY_WAITS):
     """Runs one CTA's units, (tiles, key blocks) each; raises Fault."""
     rng = random.Random(seed)
     now, heap, serial = 0.0, [], 0
@@ -116,6 +119,11 @@ def simulate(units, ks, vs, seed):
                 then = [pv_done[x][b]] + [v_empty[g % vs]] * (1 if two else 2)
                 product("V", g % vs, g, then + ([o_full] if i + di >= n else []))
                 products[uc] += 1
+            if i0 >= n:
+                at(max(pipe, now), q_empty.arrive)
+                if empty_waits:
+                    yield o_free, (uc & 1) ^ 1
+                at(max(pipe, now), o_full.arrive)
             g0 += n
 
     def softmax(x):
@@ -167,6 +175,7 @@ UNITS = {
     "one tile, odd": [(1, 13), (1, 7), (1, 31), (1, 3), (1, 2)],
     "two tiles": [(2, 13), (2, 6), (2, 2)],
     "both": [(2, 13), (1, 13), (2, 5), (1, 8), (1, 21), (2, 2), (1, 17)],
+    "single blocks": [(1, 9), (1, 1), (1, 1), (2, 4), (1, 1), (2, 1), (1, 1), (1, 2), (1, 1)],
 }
 
 
@@ -183,3 +192,9 @@ def test_the_model_sees_rings_of_odd_depth(ks, vs):
     with pytest.raises(Fault):
         for seed in range(400):
             simulate(UNITS["one tile"], ks, vs, seed)
+
+
+def test_the_model_sees_a_stream_without_a_block_that_does_not_wait():
+    with pytest.raises(Fault):
+        for seed in range(400):
+            simulate(UNITS["single blocks"], KS, VS, seed, empty_waits=False)
