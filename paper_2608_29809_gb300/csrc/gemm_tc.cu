@@ -193,12 +193,18 @@ __device__ __forceinline__ void store_bf16(bf16* p, const float* v) {
   }
 }
 
-// The gated residual of one warp's 32 x 32 chunk (lane = row, v = its 32
-// columns) as vector reductions into x: each lane parks its row in the warp's
-// 4 KB staging area, then eight lanes add one whole 128-byte row piece.
+// One warp's 32 x 32 chunk (lane = row, v = its 32 columns) in f32: stored to
+// dst, or (ADD, the gated residual) as vector reductions into it.  Each lane
+// parks its row in the warp's 4 KB staging area, then eight lanes take one
+// whole 128-byte row piece: rows are n apart, so a lane's own 16-byte pieces
+// would be half sectors of 32 different rows (a caller's 4096 x 4608 x 1152
+// into f32 45.5 us that way, 34.3 this way; 9000 x 8192 x 128 147 and 72).
+// (bf16 outputs go straight from registers, see store_bf16: their pieces of 32
+// bytes are whole sectors.)
 // Staging is XOR-swizzled in 16-byte units so that both the row-per-lane
 // writes and the piece-per-lane-group reads are free of bank conflicts.
-__device__ __forceinline__ void reduce_chunk(uint8_t* stg, int lane, const float* v, float* dst) {
+template <bool ADD>
+__device__ __forceinline__ void write_chunk(uint8_t* stg, int lane, const float* v, float* dst) {
   const uint32_t s0 = saddr(stg);
 #pragma unroll
   for (int j = 0; j < 8; ++j)
@@ -214,7 +220,9 @@ __device__ __forceinline__ void reduce_chunk(uint8_t* stg, int lane, const float
     float* d = reinterpret_cast<float*>(
         __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), row));
     const float4 x = *reinterpret_cast<const float4*>(stg + row * 128 + 16 * (j ^ (row & 7)));
-    if (d) red_add_v4(d + 4 * j, x.x, x.y, x.z, x.w);
+    if (!d) continue;
+    if (ADD) red_add_v4(d + 4 * j, x.x, x.y, x.z, x.w);
+    else reinterpret_cast<float4*>(d)[j] = x;
   }
   __syncwarp();  // the staging area is rewritten by the next chunk
 }
@@ -228,16 +236,15 @@ __device__ __forceinline__ void finish_chunk(const GemmEpi& ep, int r, int M, in
                                              uint8_t* stg, int lane, const float* x0) {
   epilogue_values<MODE>(ep, c0, cl, item, v, sv);
   if (MODE == EPI_GATE_RES) {
-    reduce_chunk(stg, lane, v, r < M ? ep.xf + size_t(r) * ep.ld_xf + c0 : nullptr);
+    write_chunk<true>(stg, lane, v, r < M ? ep.xf + size_t(r) * ep.ld_xf + c0 : nullptr);
+    return;
+  }
+  if (MODE == EPI_F32) {  // (a caller's matrix: 16-byte aligned)
+    write_chunk<false>(stg, lane, v, r < M ? ep.out_f + size_t(r) * ep.ld_out + c0 : nullptr);
     return;
   }
   if (r >= M) return;
-  if (MODE == EPI_F32) {  // (a caller's matrix: 16-byte aligned)
-    float4* d = reinterpret_cast<float4*>(ep.out_f + size_t(r) * ep.ld_out + c0);
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      d[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-  } else if (MODE == EPI_GATE_RES_CAST) {
+  if (MODE == EPI_GATE_RES_CAST) {
     float* x = ep.xf + size_t(r) * ep.ld_xf + c0;
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] += x0[i];
