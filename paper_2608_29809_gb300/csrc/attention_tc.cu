@@ -190,7 +190,7 @@ __device__ __forceinline__ int query_tiles(const RowMap& rm, int n_items, int D)
 constexpr int PLAN_TABLE = 160, MAX_SPLIT = 9;
 struct PlanTable {
   uint16_t cost[2][PLAN_TABLE];
-  uint8_t split[2][PLAN_TABLE];  // 0: not tabulated
+  uint8_t split[2][PLAN_TABLE];
 };
 // Estimated duration in units of 10 ns, fitted to launches of 39 .. 4096
 // queries over 131 .. 16384 keys with every split: a block of 80 keys takes
@@ -210,11 +210,11 @@ int plan_cost(int pairs, int nkb, int grid, int tiles, int split) {
   return pairs / grid * (nkb * block + UNIT) + (nkb + split - 1) / split * block + UNIT +
          (tiles == 2 ? MERGE2 + MERGE_SHARE2 * split : MERGE1 + MERGE_SHARE1 * split);
 }
-int pick_split(int pairs, int nkb, int grid, int tiles, int* cost) {
+int pick_split(int pairs, int nkb, int grid, int tiles, int most, int* cost) {
   int best = 1;
   *cost = plan_cost(pairs, nkb, grid, tiles, 1);
   const int rest = pairs % grid;
-  for (int s = 2; s <= MAX_SPLIT && s <= nkb && rest > 0 && rest * s <= grid; ++s) {
+  for (int s = 2; s <= most && s <= nkb && rest > 0 && rest * s <= grid; ++s) {
     const int c = plan_cost(pairs, nkb, grid, tiles, s);
     if (c < *cost) {
       *cost = c;
@@ -251,7 +251,7 @@ struct AttnUnits {
     rows = 2 * BQ;
     split = 1;
     groups = query_groups(rm, n_items, D, rows);
-    if (tiles >= 1 && tiles <= PLAN_TABLE && pt.split[0][0]) {
+    if (tiles >= 1 && tiles <= PLAN_TABLE) {
       const bool one = pt.cost[0][tiles - 1] < pt.cost[1][groups - 1];
       split = one ? pt.split[0][tiles - 1] : pt.split[1][groups - 1];
       if (one) {
@@ -1428,12 +1428,14 @@ int device_sms_attn() {
 }
 
 // The plans of a (heads, keys) shape, cached.  With a capture every key sits in
-// one unit.
+// one unit, of one tile or two by the same estimate (always two, as for launches
+// past the table, left 1024 tokens on 64 SMs: the scores of 28 blocks from 200
+// text tokens and 8 of them listed 582 us, 474 now).
 PlanTable plan_table(int heads, int Nk, int grid, bool capture) {
   static std::mutex mu;
   static std::unordered_map<uint64_t, PlanTable> cache;
-  if (capture) return PlanTable{};
-  const uint64_t key = (uint64_t(heads) << 40) | (uint64_t(grid) << 32) | uint64_t(unsigned(Nk));
+  const uint64_t key = (uint64_t(capture ? 1 : 0) << 63) | (uint64_t(heads) << 40) |
+                       (uint64_t(grid) << 32) | uint64_t(unsigned(Nk));
   std::lock_guard<std::mutex> lock(mu);
   auto it = cache.find(key);
   if (it != cache.end()) return it->second;
@@ -1441,8 +1443,8 @@ PlanTable plan_table(int heads, int Nk, int grid, bool capture) {
   for (int tiles = 1; tiles <= 2; ++tiles)
     for (int i = 0; i < PLAN_TABLE; ++i) {
       int cost;
-      t.split[tiles - 1][i] =
-          uint8_t(pick_split((i + 1) * heads, (Nk + BKV - 1) / BKV, grid, tiles, &cost));
+      t.split[tiles - 1][i] = uint8_t(pick_split((i + 1) * heads, (Nk + BKV - 1) / BKV, grid,
+                                                 tiles, capture ? 1 : MAX_SPLIT, &cost));
       t.cost[tiles - 1][i] = uint16_t(cost < 65535 ? cost : 65535);
     }
   if (cache.size() > 1024) cache.clear();
