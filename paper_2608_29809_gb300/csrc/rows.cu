@@ -147,9 +147,8 @@ mask_colstats_kernel(const float* __restrict__ A, int S, int N, int M,
 // dilation on the grid, and the compact list of dirty tokens in ascending
 // order.  CTA c owns tokens [c per, (c + 1) per), per a multiple of 32; the
 // union is a bit per token in every CTA's shared memory.
-constexpr int MASK_CTAS = 8, MASK_THREADS = 512, MASK_WARPS = MASK_THREADS / 32;
+constexpr int MASK_CTAS = 8;
 constexpr int MASK_MAX_TOKENS = 16384, MASK_WORDS = MASK_MAX_TOKENS / 32;
-constexpr int MASK_WPW = MASK_WORDS / MASK_CTAS / MASK_WARPS;  // words of a warp, at most
 
 __device__ __forceinline__ uint32_t peer_shared(const void* p, int rank) {
   uint32_t r;
@@ -165,15 +164,17 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
-template <bool FROM_MAP>
-__global__ void __launch_bounds__(MASK_THREADS, 1)
+template <bool FROM_MAP, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1)
 mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, int gw,
                     const __grid_constant__ DeltaIds ids, float tau, int r, int nblk,
                     float* __restrict__ abar, const float2* __restrict__ part,
                     uint8_t* __restrict__ mask, int32_t* __restrict__ idx,
                     int32_t* __restrict__ count) {
+  constexpr int WARPS = THREADS / 32;
+  constexpr int WPW = MASK_WORDS / MASK_CTAS / WARPS;  // words of a warp, at most
   __shared__ float s_lo[MASK_CTAS][64], s_hi[MASK_CTAS][64];  // per CTA (row 0 when not FROM_MAP)
-  __shared__ float s_wlo[64][MASK_WARPS], s_whi[64][MASK_WARPS];
+  __shared__ float s_wlo[64][FROM_MAP ? WARPS : 1], s_whi[64][FROM_MAP ? WARPS : 1];
   __shared__ float s_mn[64], s_rng[64], s_inv[64];
   __shared__ int s_ok[64];
   __shared__ uint32_t s_bits[MASK_WORDS];
@@ -187,13 +188,13 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
   pdl_trigger();
   if (FROM_MAP) {
     // a warp takes 4 x 32 tokens of one delta token at a time
-    for (int e = threadIdx.x; e < 64 * MASK_WARPS; e += MASK_THREADS) {
+    for (int e = threadIdx.x; e < 64 * WARPS; e += THREADS) {
       (&s_wlo[0][0])[e] = FLT_MAX;
       (&s_whi[0][0])[e] = -FLT_MAX;
     }
     __syncthreads();
     const int groups = (words + 3) / 4;
-    for (int u = warp; u < groups * ids.n; u += MASK_WARPS) {
+    for (int u = warp; u < groups * ids.n; u += WARPS) {
       const int j = u / groups, i = t0 + (u - j * groups) * 128 + lane;
       const float* p[4];
       float a[4];
@@ -215,9 +216,9 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
       }
     }
     __syncthreads();
-    for (int j = warp; j < ids.n; j += MASK_WARPS) {
-      float lo = lane < MASK_WARPS ? s_wlo[j][lane] : FLT_MAX;
-      float hi = lane < MASK_WARPS ? s_whi[j][lane] : -FLT_MAX;
+    for (int j = warp; j < ids.n; j += WARPS) {
+      float lo = lane < WARPS ? s_wlo[j][lane] : FLT_MAX;
+      float hi = lane < WARPS ? s_whi[j][lane] : -FLT_MAX;
       warp_bounds(lo, hi);
       if (lane < MASK_CTAS) {
         st_peer(peer_shared(&s_lo[rank][j], lane), __float_as_uint(lo));
@@ -226,7 +227,7 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
     }
     cluster_barrier();
   } else {
-    for (int j = warp; j < ids.n; j += MASK_WARPS) {
+    for (int j = warp; j < ids.n; j += WARPS) {
       float lo = FLT_MAX, hi = -FLT_MAX;
       for (int b = lane; b < nblk; b += 32) {
         const float2 v = __ldg(part + size_t(b) * ids.n + j);
@@ -262,29 +263,28 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
   // (relative), so the division is taken only where that does not settle the
   // comparison, and wherever the product is NaN
   {
-    bool u[MASK_WPW] = {};
+    bool u[WPW] = {};
     const float margin = fmaxf(1e-6f * fabsf(tau), 1e-37f);
     const float tau_hi = tau + margin, tau_lo = tau - margin;
 #pragma unroll 4
     for (int j = 0; j < ids.n; ++j) {
       const float* aj = abar + size_t(j) * N + t0 + lane;
-      float a[MASK_WPW];
+      float a[WPW];
 #pragma unroll
-      for (int q = 0; q < MASK_WPW; ++q)
-        a[q] = t0 + (warp + q * MASK_WARPS) * 32 + lane < t1 ? aj[(warp + q * MASK_WARPS) * 32]
-                                                             : 0.f;
+      for (int q = 0; q < WPW; ++q)
+        a[q] = t0 + (warp + q * WARPS) * 32 + lane < t1 ? aj[(warp + q * WARPS) * 32] : 0.f;
       const bool ok = s_ok[j];
       const float mn = s_mn[j], rng = s_rng[j], inv = s_inv[j];
 #pragma unroll
-      for (int q = 0; q < MASK_WPW; ++q)
-        if (warp + q * MASK_WARPS < words) {  // (the same for the whole warp)
+      for (int q = 0; q < WPW; ++q)
+        if (warp + q * WARPS < words) {  // (the same for the whole warp)
           const float x = __fsub_rn(a[q], mn), v = __fmul_rn(x, inv);
           u[q] |= ok && (v > tau_hi || (!(v < tau_lo) && __fdiv_rn(x, rng) >= tau));
         }
     }
 #pragma unroll
-    for (int q = 0; q < MASK_WPW; ++q) {
-      const int w = warp + q * MASK_WARPS;
+    for (int q = 0; q < WPW; ++q) {
+      const int w = warp + q * WARPS;
       if (w >= words) break;
       const uint32_t bits = __ballot_sync(0xffffffffu, u[q] && t0 + w * 32 + lane < t1);
       if (lane < MASK_CTAS) st_peer(peer_shared(&s_bits[t0 / 32 + w], lane), bits);
@@ -294,10 +294,10 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
   // dilation: any union token among the row's tokens x - r .. x + r of the
   // rows y - r .. y + r (at most 17 consecutive bits a row, in two words)
   const int nw = (N + 31) / 32;
-  uint32_t mine[MASK_WPW];  // this warp's mask words
+  uint32_t mine[WPW];  // this warp's mask words
 #pragma unroll
-  for (int q = 0; q < MASK_WPW; ++q) {
-    const int w = warp + q * MASK_WARPS, i = t0 + w * 32 + lane;
+  for (int q = 0; q < WPW; ++q) {
+    const int w = warp + q * WARPS, i = t0 + w * 32 + lane;
     bool m = false;
     if (w < words && i < t1) {
       const int y = i / gw, x = i - y * gw;
@@ -339,8 +339,8 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
     total += s_cnt[c];
   }
 #pragma unroll
-  for (int q = 0; q < MASK_WPW; ++q) {
-    const int w = warp + q * MASK_WARPS;
+  for (int q = 0; q < WPW; ++q) {
+    const int w = warp + q * WARPS;
     if (w < words && (mine[q] >> lane) & 1u)
       idx[before + s_word[w] + __popc(mine[q] & ((1u << lane) - 1u))] = t0 + w * 32 + lane;
   }
@@ -352,6 +352,11 @@ mask_cluster_kernel(const float* __restrict__ A, int S, int N, int M, int gh, in
 // 5.9 / 6.4, 16384 6.8 / 6.5, 32768 (4096 tokens) 9.4 / 8.1: eight SMs fetch
 // the scattered sectors of a larger map too slowly.
 constexpr long long MASK_CLUSTER_SCORES = 8192;
+// In the two-launch form the cluster thresholds every delta token's means on
+// eight SMs: from this many on with 32 warps each instead of 16.  Measured, 512
+// / 1024 threads, whole call: 4096 tokens 4 delta tokens 9.1 / 9.7 us, 16384
+// tokens 1 9.3 / 9.3, 8 12.7 / 11.3, 16 18.3 / 15.8, 64 53.6 / 42.9.
+constexpr int MASK_WIDE_DELTAS = 8;
 
 cudaError_t launch_localize(const float* A, int S, int N, int M, int gh, int gw,
                             const DeltaIds& ids, float tau, int dilation, uint8_t* mask,
@@ -363,9 +368,12 @@ cudaError_t launch_localize(const float* A, int S, int N, int M, int gh, int gw,
   if (!from_map)
     RC_TRY(launch_k(mask_colstats_kernel, dim3(nblk, ids.n), dim3(MASK_ROWS), 0, st, A, S, N, M,
                     ids, w.abar, w.part));
-  RC_TRY(launch_k_cluster(from_map ? mask_cluster_kernel<true> : mask_cluster_kernel<false>,
-                          dim3(MASK_CTAS), dim3(MASK_THREADS), 0, MASK_CTAS, st, A, S, N, M, gh,
-                          gw, ids, tau, dilation, nblk, w.abar, w.part, mask, idx, count));
+  const bool wide = !from_map && ids.n >= MASK_WIDE_DELTAS;
+  RC_TRY(launch_k_cluster(from_map ? mask_cluster_kernel<true, 512>
+                          : wide   ? mask_cluster_kernel<false, 1024>
+                                   : mask_cluster_kernel<false, 512>,
+                          dim3(MASK_CTAS), dim3(wide ? 1024 : 512), 0, MASK_CTAS, st, A, S, N, M,
+                          gh, gw, ids, tau, dilation, nblk, w.abar, w.part, mask, idx, count));
   count_launches(from_map ? 1 : 2);
   return cudaSuccess;
 }
