@@ -41,7 +41,6 @@
 // in a workspace (as column planes, so that accesses are whole 512-byte runs),
 // and the CTA that finishes last merges them.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 #include <math.h>
 
 #include <mutex>
@@ -50,6 +49,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "tc_common.cuh"
+#include "tma_host.h"
 
 namespace rc {
 
@@ -824,8 +824,8 @@ done:
 // S = Q K^T (M = 128, N = 128) in TMEM, an exact softmax per row (no running
 // max, no rescaling), P (bf16) written over S, O = P V (N = DHP, 8 MMAs of 16
 // keys, P read from TMEM as the A operand), O normalised and stored.  The
-// text cross-attention of a block has 120 keys: the general kernel's two
-// dependent 64-key rounds become one.
+// text cross-attention of a block has 120 keys: two dependent blocks of the
+// general kernel.
 constexpr int XK = 128;  // keys per pass
 template <int DH>
 struct XCfg {
@@ -1335,20 +1335,6 @@ xfused_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 }
 
 // ------------------------------------------------------------------- host
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  });
-  return fn;
-}
-
 struct HeadMapKey {
   const void* p;
   int rows, ld, heads, dh;
@@ -1380,7 +1366,7 @@ cudaError_t head_map(const bf16* p, int rows, int ld, int heads, int dh, int box
       return cudaSuccess;
     }
   }
-  auto fn = encode_fn();
+  auto fn = tma_encode_fn();
   if (!fn) return cudaErrorNotSupported;
   cuuint64_t dims[3] = {cuuint64_t(dh), cuuint64_t(heads), cuuint64_t(rows)};
   cuuint64_t strides[2] = {cuuint64_t(dh) * sizeof(bf16), cuuint64_t(ld) * sizeof(bf16)};
@@ -1454,10 +1440,7 @@ PlanTable plan_table(int heads, int Nk, int grid, bool capture) {
 
 }  // namespace
 
-size_t attention_split_floats(int Nmax, int heads, int dh) {
-  (void)Nmax;
-  (void)heads;
-  (void)dh;
+size_t attention_split_floats() {
   const int sms = device_sms_attn();
   return size_t(SLOTS_PER_SM) * (sms > 0 ? sms : 160) * BQ * PART_STRIDE;
 }
@@ -1465,7 +1448,6 @@ size_t attention_tickets() {
   const int sms = device_sms_attn();
   return size_t(SLOTS_PER_SM) * (sms > 0 ? sms : 160);
 }
-
 
 cudaError_t launch_attention(const bf16* Q, int ldq, const bf16* K, const bf16* V, int ldkv,
                              int kv_rows, const AttnItems& ai, int Nk, bf16* O, int ldo, int heads,

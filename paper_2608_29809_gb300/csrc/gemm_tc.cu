@@ -32,7 +32,6 @@
 // 4096 rows 177 -> 158 / 661 -> 604 us.  Two TMEM accumulators of up to 256 columns let the epilogue
 // of one tile overlap the main loop of the next.
 #include <cuda.h>
-#include <cudaTypedefs.h>
 
 #include <mutex>
 #include <unordered_map>
@@ -40,6 +39,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "tc_common.cuh"
+#include "tma_host.h"
 
 namespace rc {
 
@@ -91,13 +91,6 @@ __host__ __device__ constexpr int bmap_index(int rows) {
 }
 
 // ---------------------------------------------------------------- epilogue
-__device__ __forceinline__ void load32(const float* p, float* v) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    float4 a = __ldg(reinterpret_cast<const float4*>(p) + i);
-    v[4 * i] = a.x; v[4 * i + 1] = a.y; v[4 * i + 2] = a.z; v[4 * i + 3] = a.w;
-  }
-}
 __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, float d) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c),
                "f"(d)
@@ -710,20 +703,6 @@ GemmKernel gemm_kernel(int mode) {
 constexpr int GEMM_MODES = 6;
 
 // ------------------------------------------------------------------- host
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  });
-  return fn;
-}
-
 struct MapKey {
   const void* p;
   uint64_t rows, cols, ld;
@@ -753,7 +732,7 @@ cudaError_t tensor_map(const bf16* p, int rows, int cols, int ld, int box_rows, 
       return cudaSuccess;
     }
   }
-  auto fn = encode_fn();
+  auto fn = tma_encode_fn();
   if (!fn) return cudaErrorNotSupported;
   cuuint64_t dims[2] = {cuuint64_t(cols), cuuint64_t(rows)};
   cuuint64_t strides[1] = {cuuint64_t(ld) * sizeof(bf16)};
@@ -769,7 +748,7 @@ cudaError_t tensor_map(const bf16* p, int rows, int cols, int ld, int box_rows, 
   return cudaSuccess;
 }
 
-// Tile-width table of a GEMM shape, cached (the cost model runs up to 4 x 5
+// Tile-width table of a GEMM shape, cached (the cost model runs up to 4 x 8
 // plans per row-tile count).
 BnTable bn_table(int n, int k, int grid, int mode, int mt_bound, bool pair) {
   static std::mutex mu;

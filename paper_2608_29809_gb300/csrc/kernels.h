@@ -161,7 +161,7 @@ struct AttnScratch {
   size_t part_floats;
   unsigned* ticket;  // attention_tickets() of them, zero between launches
 };
-size_t attention_split_floats(int Nmax, int heads, int dh);
+size_t attention_split_floats();
 size_t attention_tickets();
 
 // Per-item key / value placement of one attention launch: item i's keys are

@@ -529,7 +529,7 @@ rc_status rc_create(const rc_dims* dims, rc_ctx** out) {
     free_ctx(c);
     return s;
   }
-  c->as.part_floats = rc::attention_split_floats(int(N), D.heads, dh);
+  c->as.part_floats = rc::attention_split_floats();
   if ((s = dalloc(&c->as.part, c->as.part_floats, "attn part")) ||
       (s = dalloc(&c->as.ticket, rc::attention_tickets(), "attn tickets"))) {
     free_ctx(c);
@@ -633,8 +633,8 @@ rc_status rc_cache_create(rc_ctx* c, int sessions, rc_cache** out) {
   const size_t n_text = size_t(sessions) * c->L * c->M * 2 * c->d;
   if (s == RC_OK) s = dalloc(&k->text, n_text, "text kv");
   if (s == RC_OK) s = alloc_xg(k);
-  // zero-filled: the attention reads whole 64-key blocks, and keys past a
-  // slot's end (weighted by zero) come from the next slot, which must be finite
+  // zero-filled: the attention takes values in steps of 16 keys, and those past
+  // a slot's end (weighted by zero) come from the next slot, which must be finite
   if (s == RC_OK && (cudaMemset(k->base, 0, n * sizeof(bf16)) != cudaSuccess ||
                      cudaMemset(k->text, 0, n_text * sizeof(bf16)) != cudaSuccess ||
                      cudaDeviceSynchronize() != cudaSuccess))
@@ -891,7 +891,7 @@ rc_status rc_set_text(rc_ctx* c, rc_cache* k, int s, const void* ctx_bf16, rc_st
     if (!c->lw_set[l]) return fail(RC_ERR_STATE, "weights of layer %d not set", l);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (c->M <= rc::XQ_KEYS) {
-    // every layer in one launch: 28 launches of 10.8 us before
+    // every layer in one launch
     RC_CUDA(rc::launch_text_kv(static_cast<const bf16*>(ctx_bf16), c->tl.data(), c->L,
                                c->M, c->d, k->text_kv(s, 0), c->err, st), "text kv");
   } else {

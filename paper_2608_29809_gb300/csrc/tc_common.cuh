@@ -98,17 +98,11 @@ __device__ __forceinline__ bool mbar_sleep(uint32_t bar, uint32_t parity,
     }
   }
 }
+// mbar_sleep taken by every lane of a warp; the outcome is made warp-uniform
+// so that a timeout never leaves part of a warp at a warp-wide instruction.
 __device__ __forceinline__ bool mbar_sleep_warp(uint32_t bar, uint32_t parity,
                                                 volatile int* abort_flag) {
   const bool ok = mbar_sleep(bar, parity, abort_flag);
-  return __all_sync(0xffffffffu, ok);
-}
-
-// mbar_wait taken by every lane of a warp; the outcome is made warp-uniform
-// so that a timeout never leaves part of a warp at a warp-wide instruction.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity,
-                                               volatile int* abort_flag) {
-  const bool ok = mbar_wait(bar, parity, abort_flag);
   return __all_sync(0xffffffffu, ok);
 }
 
@@ -243,8 +237,6 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t addr) {
   return d;
 }
 
-
-
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
                                             int x, int y, int z) {
   asm volatile(
@@ -260,19 +252,6 @@ __device__ __forceinline__ uint64_t sw32_kmajor_desc(uint32_t addr) {
   uint64_t d = 0;
   d |= uint64_t((addr & 0x3FFFFu) >> 4);
   d |= uint64_t(16 >> 4) << 16;
-  d |= uint64_t(256 >> 4) << 32;
-  d |= uint64_t(1) << 46;
-  d |= uint64_t(6) << 61;
-  return d;
-}
-
-// MN-major bf16 operand with the 32-byte swizzle: 16 MN-contiguous elements
-// per 32-byte row, consecutive K rows 32 B apart; `lbo` bytes between
-// 16-element MN groups, 8-row K groups 256 B apart.
-__device__ __forceinline__ uint64_t sw32_mnmajor_desc(uint32_t addr, uint32_t lbo) {
-  uint64_t d = 0;
-  d |= uint64_t((addr & 0x3FFFFu) >> 4);
-  d |= uint64_t((lbo >> 4) & 0x3FFFu) << 16;
   d |= uint64_t(256 >> 4) << 32;
   d |= uint64_t(1) << 46;
   d |= uint64_t(6) << 61;
