@@ -39,10 +39,8 @@ static inline int row_grid(int rows_bound, int rows_per_cta, int per_sm) {
 // cluster of eight CTAs shares the column bounds, the thresholded region and
 // the counts through its shared memory, so that the steps that need every
 // token's result of the previous one are cluster barriers instead of
-// launches.  1024 tokens, 5 delta tokens: 7.9 -> 5.9 us on the device (four
-// launches before), 17.9 -> 12.6 us a call from Python (8.3 since the binding
-// asks for the raw stream handle); 16384 tokens, 8 delta tokens, 16 slices:
-// 50 -> 32 us.
+// launches.  1024 tokens, 5 delta tokens: 5.9 us on the device (7.9 with four
+// launches); 16384 tokens, 8 delta tokens, 16 slices: 30.9 us a call (50).
 // Workspace: abar f32 [n_delta][N] | part f32x2 [nblk][n_delta] | union u8 [N]
 // | cnt int [nblk] (the last two are unused and kept for the stated size).
 constexpr int MASK_ROWS = 256;
